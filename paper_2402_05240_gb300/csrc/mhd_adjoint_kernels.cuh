@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(BX* BY) k_adj_floors(Grid g, const double* __r
   double gb[3] = {0.0, 0.0, 0.0};
   const bool rfl = u5[0] < g.rho_floor;
   const double r = rfl ? g.rho_floor : u5[0];
-  const double ir = __drcp_rn(r);
+  const double ir = trcp<double>(r);
   // kinetic + magnetic energy and the pressure-floor test with the forward's
   // arithmetic (k_prim; its FP32-bulk form in p_recover_f32)
   double ke, me;

@@ -15,6 +15,7 @@
 #include <stdint.h>
 
 #include "mhd_df.cuh"
+#include "mhd_int53.cuh"
 #include "mhd_launch.h"
 
 namespace mhd {
@@ -35,16 +36,16 @@ __device__ __forceinline__ long long nb(const Grid& g, int i, int j, int k, int 
 }
 
 template <class T> __device__ __forceinline__ T tsqrt(T x);
-template <> __device__ __forceinline__ double tsqrt<double>(double x) { return sqrt(x); }
+template <> __device__ __forceinline__ double tsqrt<double>(double x) { return sqrt_int(x); }
 template <> __device__ __forceinline__ float tsqrt<float>(float x) { return sqrtf(x); }
 
-// correctly rounded reciprocal (cheaper than a general division) and the
-// library reciprocal square root
+// correctly rounded reciprocal (cheaper than a general division) and
+// reciprocal square root; double: on the integer pipes (mhd_int53.cuh)
 template <class T> __device__ __forceinline__ T trcp(T x);
-template <> __device__ __forceinline__ double trcp<double>(double x) { return __drcp_rn(x); }
+template <> __device__ __forceinline__ double trcp<double>(double x) { return rcp_int(x); }
 template <> __device__ __forceinline__ float trcp<float>(float x) { return __frcp_rn(x); }
 template <class T> __device__ __forceinline__ T trsqrt(T x);
-template <> __device__ __forceinline__ double trsqrt<double>(double x) { return rsqrt(x); }
+template <> __device__ __forceinline__ double trsqrt<double>(double x) { return rsqrt_int(x); }
 template <> __device__ __forceinline__ float trsqrt<float>(float x) { return rsqrtf(x); }
 
 template <> __device__ __forceinline__ df tsqrt<df>(df x) { return df_sqrt(x); }

@@ -170,7 +170,7 @@ __device__ __forceinline__ PrimD prim_core_ir(const Grid& g, double rho, double 
 __device__ __forceinline__ PrimD prim_core(const Grid& g, double r, double m0, double m1, double m2, double e,
                                            const double* b) {
   const double rho = max_pos<double>(r, g.rho_floor);
-  return prim_core_ir(g, rho, __drcp_rn(rho), m0, m1, m2, e, b);
+  return prim_core_ir(g, rho, trcp<double>(rho), m0, m1, m2, e, b);
 }
 
 // Cell-centred reference electric field E = -(v x B_cc) of one cell (Sec. 2.2
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(BX* BY) k_prim(Grid g, Fields<double, 8> U, Fi
       if (in) atomicAdd(&floors[0], 1ull);
     }
     const double rho = max_pos<double>(r, g.rho_floor);
-    const double ir = __drcp_rn(rho);
+    const double ir = trcp<double>(rho);
     T w8[8];
     if constexpr (std::is_same<T, float>::value) {
       const double bs[3] = {b0m + b0p, b1m + b1p, b2m + b2p};
@@ -772,7 +772,7 @@ __global__ void __launch_bounds__(BX* BY) k_update_half(Grid g, Fields<const dou
     const double bs[3] = {bxm + bx, bym + by, bzm + bz};
     const double rho = max_pos<double>(u5[0], g.rho_floor);
     double t2, pg;
-    prim_store_f32(g, W, c, rho, __drcp_rn(rho), u5[1], u5[2], u5[3], u5[4], bs, w8, t2, pg);
+    prim_store_f32(g, W, c, rho, trcp<double>(rho), u5[1], u5[2], u5[3], u5[4], bs, w8, t2, pg);
   } else {
     const double bcc[3] = {0.5 * (bxm + bx), 0.5 * (bym + by), 0.5 * (bzm + bz)};
     const PrimD pw = prim_core(g, u5[0], u5[1], u5[2], u5[3], u5[4], bcc);
