@@ -122,6 +122,45 @@ template <> __device__ __forceinline__ double max_s<double>(double x, double y) 
   return dkey(x) < dkey(y) ? y : x;
 }
 
+template <class T> __device__ __forceinline__ T neg(T x) { return -x; }
+template <> __device__ __forceinline__ double neg<double>(double x) { return __longlong_as_double(dbits(x) ^ kNegZero); }
+// Scalings by 2, 4 and 1/2.  Double: on the bit pattern.  twice() serves the
+// limiters (finite normal operands or zeros, no overflow); half() is exact for
+// every operand but odd subnormals (cut by half the smallest one); quad()
+// falls back to the multiplication, executed only in warps where a lane needs
+// it, where operand or result is not normal.
+template <class T> __device__ __forceinline__ T twice(T x) { return T(2) * x; }
+template <> __device__ __forceinline__ df twice<df>(df x) { return df(2.0f * x.hi, 2.0f * x.lo); }
+template <> __device__ __forceinline__ double twice<double>(double v) {
+  const long long x = dbits(v);
+  return (x & kAbsBits) ? __longlong_as_double(x + (1LL << 52)) : v;
+}
+template <class T> __device__ __forceinline__ T half(T x) { return T(0.5) * x; }
+template <> __device__ __forceinline__ df half<df>(df x) { return df(0.5f * x.hi, 0.5f * x.lo); }
+template <> __device__ __forceinline__ double half<double>(double x) {
+  const long long b = dbits(x), m = b & kAbsBits;
+  const long long small = (m >> 1) | (b & kNegZero);  // operand or result not normal
+  const long long r = m < (2LL << 52) ? small : b - (1LL << 52);
+  return __longlong_as_double(m >= 0x7ff0000000000000LL ? b : r);
+}
+template <class T> __device__ __forceinline__ T quad(T x) { return T(4) * x; }
+template <> __device__ __forceinline__ df quad<df>(df x) { return df(4.0f * x.hi, 4.0f * x.lo); }
+template <> __device__ __forceinline__ double quad<double>(double x) {
+  const int hi = __double2hiint(x);
+  const bool fast = (unsigned)(hi & 0x7fffffff) - 0x00100000u < 0x7fd00000u - 0x00100000u;
+  double r = __hiloint2double(hi + 0x00200000, __double2loint(x));
+  if (__any_sync(__activemask(), !fast)) {
+    if (!fast) r = 4.0 * x;
+  }
+  return r;
+}
+// s x for s = +-1 (a sign flip for double and float pairs)
+template <class T> __device__ __forceinline__ T times_sign(T x, T s) { return x * s; }
+template <> __device__ __forceinline__ df times_sign<df>(df x, df s) { return s.hi < 0.0f ? df(-x.hi, -x.lo) : x; }
+template <> __device__ __forceinline__ double times_sign<double>(double x, double s) {
+  return __longlong_as_double(dbits(x) ^ (dbits(s) & kNegZero));
+}
+
 // Conversions between the compute type and double without the conversion
 // instructions, which issue at the FP64 rate on this GPU (mhd_df.cuh).
 template <class T> __device__ __forceinline__ double to_d(T x);
@@ -175,8 +214,24 @@ __device__ __forceinline__ T fast_speed(T gamma, T rho, T p, T bl, T bt1, T bt2)
 // bn = longitudinal face field.  Outer speeds S_L = min(u) - max(c_f),
 // S_R = max(u) + max(c_f); degenerate star / double-star states below
 // Eps<T>::hlld * p_T*; flux selection with ties to the left.  gm1i = 1/(gamma - 1).
+//
+// Double and float pairs (hlld_diff): every increment of F + S (U* - U) +
+// S* (U** - U*) is formed from the differences that cause it.  With delta =
+// S_M - u = (rho'(S' - u')(u_R - u_L) + p_L - p_R) / den (primes: the other
+// side), t = B_n delta / D and q - 1 = rho (S - u) delta / D, the star
+// increments are rho* - rho = rho delta / (S - S_M), v* - v = -B_t t, B* - B_t =
+// B_t (q - 1), and the double-star ones share one velocity difference.  That
+// takes 90 operations where no lane of the warp lies between the Alfven waves
+// and 132 where one does, against 156 in the jump form; equal states give
+// their physical flux exactly, and the degenerate limit is delta / D = 0.
+// The other side's star state is formed for double-star faces alone.  Both
+// types are bound by the arithmetic (FP64 pipe, issue slots): against the
+// jump form the PLMC step went from 72.1 to 61.8 ms (FP64, 256^3) and from
+// 116.4 to 104.7 ms (float pairs, 459^3).
+// float (hlld_jump): kept in the jump form, whose rounding fixes the
+// FP32-bulk mode's results.
 template <class T>
-__device__ __forceinline__ void hlld(T gamma, T gm1i, const T* wl, const T* wr, T bn, T* f) {
+__device__ __forceinline__ void hlld_jump(T gamma, T gm1i, const T* wl, const T* wr, T bn, T* f) {
   const T bn2 = bn * bn;
   // total pressures of both sides; the conserved energy is formed only for
   // the side whose states the flux is taken from
@@ -312,6 +367,118 @@ __device__ __forceinline__ void hlld(T gamma, T gm1i, const T* wl, const T* wr, 
   }
 }
 
+template <class T>
+__device__ __forceinline__ void hlld_diff(T gamma, T gm1i, const T* wl, const T* wr, T bn, T* f) {
+  const T bn2 = bn * bn;
+  const T btL = wl[5] * wl[5] + wl[6] * wl[6], btR = wr[5] * wr[5] + wr[6] * wr[6];
+  const T bbL = bn2 + btL, bbR = bn2 + btR;
+  const T ptL = wl[4] + half<T>(bbL), ptR = wr[4] + half<T>(bbR);
+  // 2 rho c_f^2 = gamma P + B^2 + sqrt((gamma P - B^2)^2 + 4 gamma P B_t^2):
+  // no division; the larger c_f^2 is chosen by cross-multiplication, and only
+  // its side takes a reciprocal and a root
+  auto two_rho_cf2 = [&](T p, T bb, T bt) {
+    const T gp = gamma * p;
+    const T dd = gp - bb;
+    return gp + bb + tsqrt<T>(dd * dd + quad<T>(gp) * bt);
+  };
+  const T XL = two_rho_cf2(wl[4], bbL, btL), XR = two_rho_cf2(wr[4], bbR, btR);
+  const bool lmax = !nonneg_lt<T>(XL * wr[0], XR * wl[0]);
+  const T cmax = tsqrt<T>(half<T>(lmax ? XL : XR) * trcp<T>(lmax ? wl[0] : wr[0]));
+  const T SL = min_s<T>(wl[1], wr[1]) - cmax;
+  const T SR = max_s<T>(wl[1], wr[1]) + cmax;
+  const bool sub = !ge0<T>(SL) && !le0<T>(SR);
+  T rdL = T(0), rdR = T(0), dlL = T(0), dlR = T(0), SM = T(0), pts = T(0);
+  if (sub) {
+    rdL = wl[0] * (SL - wl[1]);
+    rdR = wr[0] * (SR - wr[1]);
+    const T iden = trcp<T>(rdR - rdL);
+    const T du = wr[1] - wl[1], dp = ptL - ptR;
+    dlL = (rdR * du + dp) * iden;  // S_M - u of both sides
+    dlR = (rdL * du + dp) * iden;
+    SM = wl[1] + dlL;
+    pts = ptL + rdL * dlL;
+  }
+  // the side whose states the flux is taken from (ties to the left)
+  const bool left = sub ? ge0<T>(SM) : ge0<T>(SL);
+  const T* w = left ? wl : wr;
+  const T r = w[0], u = w[1], v = w[2], vw = w[3], by = w[5], bz = w[6];
+  const T pt = left ? ptL : ptR, bt = left ? btL : btR;
+  const T e = w[4] * gm1i + (half<T>(r) * (u * u + v * v + vw * vw) + half<T>(left ? bbL : bbR));
+  const T mu = r * u;
+  const T vby = v * by + vw * bz;
+  // the increments S (U* - U) of the star region: zero for a supersonic face
+  T m1 = T(0), sm1 = T(0), C = bn, A = u, dE = T(0);
+  T rs = T(0), z = T(0), rd = T(0), Ss = T(0);
+  bool inner = false;
+  if (sub) {
+    const T S = left ? SL : SR, dl = left ? dlL : dlR;
+    rd = left ? rdL : rdR;
+    const T Sd = S - SM;
+    const T iSd = trcp<T>(Sd);
+    rs = rd * iSd;
+    const T D = rd * Sd - bn2;
+    // (the degenerate limit keeps the transverse state: z = 0)
+    z = abs_lt<T>(D, Eps<T>::hlld * pts) ? T(0) : dl * trcp<T>(D);
+    const T t = bn * z, rz = rd * z;  // v* = v - B_t t, B* = B_t (1 + rz)
+    // (a density jump below the rounding of rho* is none: the mass flux then
+    // keeps the sign of the resolved velocity, which the edge fields upwind by)
+    m1 = rs == r ? T(0) : S * (r * (dl * iSd));
+    sm1 = S * (rs * SM - mu);
+    C = bn + S * rs * t;
+    A = u + S * rz;
+    const T ps = pt + rd * dl;
+    const T bbt = bt * t;
+    const T dvb = rz * (vby - bbt) + (bn * dl - bbt);  // v*.B* - v.B
+    dE = S * (((e + ps + u * rd) * dl - bn * dvb) * iSd);
+    const T cA = fabs(bn) * trsqrt<T>(rs);
+    Ss = left ? SM - cA : SM + cA;
+    inner = (left ? lt0<T>(Ss) : ge0<T>(Ss)) && !nonneg_lt<T>(half<T>(bn2), Eps<T>::hlld * pts);
+  }
+  const T f0 = mu + m1;
+  f[0] = f0;
+  f[1] = mu * u + (pt - bn2) + sm1;
+  f[2] = f0 * v - by * C;
+  f[3] = f0 * vw - bz * C;
+  f[4] = (e + pt) * u - bn * (u * bn + vby) + dE;
+  f[5] = by * A - bn * v;
+  f[6] = bz * A - bn * vw;
+  if (inner) {
+    // the increments Ss (U** - U*) of the double-star region: with the star
+    // states of both sides, Delta = v** - v* = (sgn(B_n) (B*_R - B*_L) +-
+    // sqrt(rho*') (v*_R - v*_L)) / (sqrt(rho*_L) + sqrt(rho*_R)), rho*' the
+    // other side's, + on the left, and B** - B* = g Delta, g = +- sqrt(rho*)
+    // sgn(B_n), + on the left
+    const T* wo = left ? wr : wl;
+    const T rdo = left ? rdR : rdL;
+    const T Sdo = (left ? SR : SL) - SM;
+    const T rso = rdo * trcp<T>(Sdo);
+    const T Do = rdo * Sdo - bn2;
+    const T zo = abs_lt<T>(Do, Eps<T>::hlld * pts) ? T(0) : (left ? dlR : dlL) * trcp<T>(Do);
+    const T t = bn * z, q = T(1) + rd * z;
+    const T to = bn * zo, qo = T(1) + rdo * zo;
+    const T vs = v - by * t, ws = vw - bz * t, bys = by * q, bzs = bz * q;
+    const T sq = rs * trsqrt<T>(rs), sqo = rso * trsqrt<T>(rso);
+    const T inv = trcp<T>(sq + sqo);
+    const T sg = (gt0<T>(bn) == left) ? T(1) : T(-1);
+    // (differences other minus own: both terms change sign with the side)
+    const T Dy = (times_sign<T>(wo[5] * qo - bys, sg) + sqo * ((wo[2] - wo[5] * to) - vs)) * inv;
+    const T Dz = (times_sign<T>(wo[6] * qo - bzs, sg) + sqo * ((wo[3] - wo[6] * to) - ws)) * inv;
+    const T g = times_sign<T>(sq, sg);
+    const T ay = Ss * Dy, az = Ss * Dz;
+    f[2] = f[2] + rs * ay;
+    f[3] = f[3] + rs * az;
+    f[4] = f[4] + g * (ay * (bys + g * (vs + Dy)) + az * (bzs + g * (ws + Dz)));
+    f[5] = f[5] + g * ay;
+    f[6] = f[6] + g * az;
+  }
+}
+
+template <class T>
+__device__ __forceinline__ void hlld(T gamma, T gm1i, const T* wl, const T* wr, T bn, T* f) {
+  if constexpr (sizeof(T) == 4) hlld_jump<T>(gamma, gm1i, wl, wr, bn, f);
+  else hlld_diff<T>(gamma, gm1i, wl, wr, bn, f);
+}
+
 // ------------------------------------------------ characteristic projection --
 // Primitive eigen-system (rho, u, v, w, P, B_t1, B_t2) of one cell with its
 // cell-centred longitudinal field bn.  Waves ordered u-cf, u-ca, u-cs, u,
@@ -431,8 +598,6 @@ template <class T> __device__ __forceinline__ T min_abs(T a, T b) { return fmin(
 // sgn0(s) m for m >= 0
 template <class T> __device__ __forceinline__ T with_sign(T s, T m) { return sgn0<T>(s) * m; }
 template <class T> __device__ __forceinline__ bool abs_ge_twice(T a, T b) { return fabs(a) >= T(2) * fabs(b); }
-template <class T> __device__ __forceinline__ T twice(T x) { return T(2) * x; }
-template <> __device__ __forceinline__ df twice<df>(df x) { return df(2.0f * x.hi, 2.0f * x.lo); }
 
 template <> __device__ __forceinline__ bool pos_prod<double>(double a, double b) {
   const long long x = dbits(a), y = dbits(b);
@@ -454,10 +619,6 @@ template <> __device__ __forceinline__ double with_sign<double>(double s, double
 template <> __device__ __forceinline__ bool abs_ge_twice<double>(double a, double b) {
   const long long x = dbits(a) & kAbsBits, y = dbits(b) & kAbsBits;
   return x >= (y ? y + (1LL << 52) : 0LL);
-}
-template <> __device__ __forceinline__ double twice<double>(double v) {
-  const long long x = dbits(v);
-  return (x & kAbsBits) ? __longlong_as_double(x + (1LL << 52)) : v;
 }
 
 // ------------------------------------------------------- PLMC (Sec. 2.2.6) --
@@ -605,8 +766,6 @@ template <> __device__ __forceinline__ double ratio_le1<double>(double a, double
 // multiplied, and sign flips and doublings are exact bit operations, so
 // only the arithmetic the limiter needs reaches the FP64 pipe.  Same values
 // as the formulas with q[2] kept, up to the sign of zero results.
-template <class T> __device__ __forceinline__ T neg(T x) { return -x; }
-template <> __device__ __forceinline__ double neg<double>(double x) { return __longlong_as_double(dbits(x) ^ kNegZero); }
 template <class T> __device__ __forceinline__ void ppm_one(const T* q, T& qm, T& qp) {
   const T c7 = from_d<T>(7.0 / 12.0), c1 = from_d<T>(1.0 / 12.0), c6 = from_d<T>(1.0 / 6.0);
   const T a = q[0], b = q[1], d = q[3], e = q[4];  // cells i-2, i-1, i+1, i+2
