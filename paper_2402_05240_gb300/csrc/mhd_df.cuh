@@ -103,36 +103,68 @@ __device__ __forceinline__ df df_from_double(double x) {
 
 __device__ __forceinline__ df::df(double x) : df(df_from_double(x)) {}
 
+// The transformations use the intrinsics that are never merged into a fused
+// multiply-add: a product taken up by the sum that consumes it would bring its
+// rounding error in twice.
 // s + e = a + b exactly (no ordering assumed)
 __device__ __forceinline__ df two_sum(float a, float b) {
-  const float s = a + b;
-  const float v = s - a;
-  const float e = (a - (s - v)) + (b - v);
+  const float s = __fadd_rn(a, b);
+  const float v = __fsub_rn(s, a);
+  const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
   return df(s, e);
 }
 // s + e = a + b exactly when |a| >= |b| (or a == 0)
 __device__ __forceinline__ df fast_two_sum(float a, float b) {
-  const float s = a + b;
-  return df(s, b - (s - a));
+  const float s = __fadd_rn(a, b);
+  return df(s, __fsub_rn(b, __fsub_rn(s, a)));
 }
 // p + e = a * b exactly
 __device__ __forceinline__ df two_prod(float a, float b) {
-  const float p = a * b;
+  const float p = __fmul_rn(a, b);
   return df(p, fmaf(a, b, -p));
 }
 
-__device__ __forceinline__ df operator+(df x, df y) {
-  const df s = two_sum(x.hi, y.hi);
-  return fast_two_sum(s.hi, s.lo + (x.lo + y.lo));
+// Sums and products of float pairs leave their result as a pair (hi, lo) that
+// is not yet normalised: lo may reach a few ulps of hi (more after a
+// cancellation).  A further addition takes it as it stands (TwoSum is exact
+// whatever the ordering, and the low parts only add up); a multiplication, a
+// comparison, a division, a root or an assignment to a df normalises it first
+// (FastTwoSum, 3 operations).  So a sum of n products normalises once instead
+// of 2 n - 1 times -- a b + c d + e takes 27 operations instead of 36 -- with
+// the same values in hi + lo up to the rounding of the low parts.  Measured: the
+// double-float PPMC step at 512^3 went from 182 to 168 ms, with a step's error
+// against 64 bits at 1.7e-15 to 1.9e-15 (2.0e-15 before the difference-form
+// Riemann solver).
+struct dfx {
+  float hi, lo;
+  __device__ __forceinline__ dfx(float h, float l) : hi(h), lo(l) {}
+  __device__ __forceinline__ operator df() const { return fast_two_sum(hi, lo); }
+  __device__ __forceinline__ explicit operator double() const { return (double)(df)*this; }
+};
+__device__ __forceinline__ dfx df_sum(float xh, float xl, float yh, float yl) {
+  const df s = two_sum(xh, yh);
+  return dfx(s.hi, __fadd_rn(s.lo, __fadd_rn(xl, yl)));
 }
+__device__ __forceinline__ dfx operator+(df x, df y) { return df_sum(x.hi, x.lo, y.hi, y.lo); }
+__device__ __forceinline__ dfx operator+(dfx x, df y) { return df_sum(x.hi, x.lo, y.hi, y.lo); }
+__device__ __forceinline__ dfx operator+(df x, dfx y) { return df_sum(x.hi, x.lo, y.hi, y.lo); }
+__device__ __forceinline__ dfx operator+(dfx x, dfx y) { return df_sum(x.hi, x.lo, y.hi, y.lo); }
 __device__ __forceinline__ df operator-(df x) { return df(-x.hi, -x.lo); }
-__device__ __forceinline__ df operator-(df x, df y) { return x + (-y); }
-__device__ __forceinline__ df operator*(df x, df y) {
-  df p = two_prod(x.hi, y.hi);
+__device__ __forceinline__ dfx operator-(dfx x) { return dfx(-x.hi, -x.lo); }
+__device__ __forceinline__ dfx operator-(df x, df y) { return df_sum(x.hi, x.lo, -y.hi, -y.lo); }
+__device__ __forceinline__ dfx operator-(dfx x, df y) { return df_sum(x.hi, x.lo, -y.hi, -y.lo); }
+__device__ __forceinline__ dfx operator-(df x, dfx y) { return df_sum(x.hi, x.lo, -y.hi, -y.lo); }
+__device__ __forceinline__ dfx operator-(dfx x, dfx y) { return df_sum(x.hi, x.lo, -y.hi, -y.lo); }
+__device__ __forceinline__ dfx operator*(df x, df y) {
+  const df p = two_prod(x.hi, y.hi);
   float l = fmaf(x.hi, y.lo, p.lo);
   l = fmaf(x.lo, y.hi, l);
-  return fast_two_sum(p.hi, l);
+  return dfx(p.hi, l);
 }
+// the normalised forms (the exact increments of the FP32-bulk update are kept
+// in them: one rounding per operation)
+__device__ __forceinline__ df add_n(df x, df y) { return x + y; }
+__device__ __forceinline__ df mul_n(df x, df y) { return x * y; }
 __device__ __forceinline__ df operator/(df x, df y) {
   // below 2^-100 the reciprocal of the leading float would overflow for
   // subnormal divisors: scale both operands by 2^100 (exact)
@@ -148,7 +180,9 @@ __device__ __forceinline__ df operator/(df x, df y) {
   return fast_two_sum(q1, q2);
 }
 __device__ __forceinline__ df& operator+=(df& x, df y) { return x = x + y; }
+__device__ __forceinline__ df& operator+=(df& x, dfx y) { return x = x + y; }
 __device__ __forceinline__ df& operator-=(df& x, df y) { return x = x - y; }
+__device__ __forceinline__ df& operator-=(df& x, dfx y) { return x = x - y; }
 __device__ __forceinline__ df& operator*=(df& x, df y) { return x = x * y; }
 
 __device__ __forceinline__ bool operator<(df a, df b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }

@@ -653,7 +653,7 @@ __device__ __forceinline__ double face_curl(const Grid& g, const Fields<const T,
   if constexpr (EXACT && std::is_same<T, float>::value) {
     const df dc = two_sum(ldg(EC + q), -ldg(EC + q + oB));
     const df db = two_sum(ldg(EB + q), -ldg(EB + q + oC));
-    return (double)(dc * df(g.id[B]) - db * df(g.id[C]));
+    return (double)add_n(mul_n(dc, df(g.id[B])), -mul_n(db, df(g.id[C])));
   } else if (EXACT) {
     return (to_d<T>(ldg(EC + q)) - to_d<T>(ldg(EC + q + oB))) * g.id[B] -
            (to_d<T>(ldg(EB + q)) - to_d<T>(ldg(EB + q + oC))) * g.id[C];
@@ -701,7 +701,7 @@ __device__ __forceinline__ void hydro_update(const Fields<const double, 8>& U0, 
       for (int a = 0; a < 3; ++a) {
         const T* Fa = F.f[a * 7 + comp_of(f, a)];
         const df hdf = HALF ? df(S.hd_half_hi[a], S.hd_half_lo[a]) : df(S.hd_full_hi[a], S.hd_full_lo[a]);
-        inc += hdf * two_sum(ldg(Fa + c), -ldg(Fa + c + p.m[a]));
+        inc = add_n(inc, mul_n(hdf, two_sum(ldg(Fa + c), -ldg(Fa + c + p.m[a]))));
       }
       out5[f] = ldu<NC>(U0.f[f] + c) - (double)inc;
     } else if (EXACT) {
