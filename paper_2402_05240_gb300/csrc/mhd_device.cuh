@@ -154,6 +154,15 @@ template <> __device__ __forceinline__ double quad<double>(double x) {
   }
   return r;
 }
+// x / 4; as half()
+template <class T> __device__ __forceinline__ T quarter(T x) { return T(0.25) * x; }
+template <> __device__ __forceinline__ df quarter<df>(df x) { return df(0.25f * x.hi, 0.25f * x.lo); }
+template <> __device__ __forceinline__ double quarter<double>(double x) {
+  const long long b = dbits(x), m = b & kAbsBits;
+  const long long small = (m >> 2) | (b & kNegZero);  // zero; operand or result not normal
+  const long long r = m < (3LL << 52) ? small : b - (2LL << 52);
+  return __longlong_as_double(m >= 0x7ff0000000000000LL ? b : r);
+}
 // s x for s = +-1 (a sign flip for double and float pairs)
 template <class T> __device__ __forceinline__ T times_sign(T x, T s) { return x * s; }
 template <> __device__ __forceinline__ df times_sign<df>(df x, df s) { return s.hi < 0.0f ? df(-x.hi, -x.lo) : x; }
@@ -167,6 +176,10 @@ template <class T> __device__ __forceinline__ double to_d(T x);
 template <> __device__ __forceinline__ double to_d<double>(double x) { return x; }
 template <> __device__ __forceinline__ double to_d<float>(float x) { return f2d_bits(x); }
 template <> __device__ __forceinline__ double to_d<df>(df x) { return (double)x; }
+// the nearest float (float pairs: the leading one)
+template <class T> __device__ __forceinline__ float to_f(T x);
+template <> __device__ __forceinline__ float to_f<double>(double x) { return d2f_bits(x); }
+template <> __device__ __forceinline__ float to_f<df>(df x) { return x.hi; }
 template <class T> __device__ __forceinline__ T from_d(double x);
 template <> __device__ __forceinline__ double from_d<double>(double x) { return x; }
 template <> __device__ __forceinline__ float from_d<float>(double x) { return d2f_bits(x); }

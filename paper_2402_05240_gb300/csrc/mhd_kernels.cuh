@@ -150,9 +150,10 @@ template <class T> __device__ __forceinline__ T cell_inv_crossing(const Grid& g,
 }
 
 // primitives from a double state of one cell: rho' = max(rho, floor),
-// v = m / rho', P' = max((gamma-1)(E - m.v/2 - |B_cc|^2/2), floor)
+// v = m / rho', P' = max((gamma-1)(E - (m.v + |B_cc|^2)/2), floor).  t2 = m.v +
+// |B_cc|^2 and pg, the pressure before the floor, serve the floor reset.
 __device__ __forceinline__ PrimD prim_core_ir(const Grid& g, double rho, double ir, double m0, double m1, double m2,
-                                              double e, const double* b) {
+                                              double e, const double* b, double& t2, double& pg) {
   PrimD w;
   w.b[0] = b[0];
   w.b[1] = b[1];
@@ -161,16 +162,17 @@ __device__ __forceinline__ PrimD prim_core_ir(const Grid& g, double rho, double 
   w.v[0] = m0 * ir;
   w.v[1] = m1 * ir;
   w.v[2] = m2 * ir;
-  const double ke = 0.5 * (m0 * w.v[0] + m1 * w.v[1] + m2 * w.v[2]);
-  const double me = 0.5 * (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
-  w.p = max_pos<double>(g.gm1 * (e - ke - me), g.p_floor);
+  t2 = (m0 * w.v[0] + m1 * w.v[1] + m2 * w.v[2]) + (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
+  pg = g.gm1 * (e - 0.5 * t2);
+  w.p = max_pos<double>(pg, g.p_floor);
   return w;
 }
 
 __device__ __forceinline__ PrimD prim_core(const Grid& g, double r, double m0, double m1, double m2, double e,
                                            const double* b) {
   const double rho = max_pos<double>(r, g.rho_floor);
-  return prim_core_ir(g, rho, trcp<double>(rho), m0, m1, m2, e, b);
+  double t2, pg;
+  return prim_core_ir(g, rho, trcp<double>(rho), m0, m1, m2, e, b, t2, pg);
 }
 
 // Cell-centred reference electric field E = -(v x B_cc) of one cell (Sec. 2.2
@@ -179,6 +181,7 @@ __device__ __forceinline__ PrimD prim_core(const Grid& g, double r, double m0, d
 // cell, so the edge fields read one value per cell instead of four primitives.
 template <class T, int A> __device__ __forceinline__ T cell_ref(const T* w8) {
   constexpr int B = (A + 1) % 3, C = (A + 2) % 3;
+  if constexpr (sizeof(T) != 4) return w8[1 + C] * w8[5 + B] - w8[1 + B] * w8[5 + C];
   return -(w8[1 + B] * w8[5 + C] - w8[1 + C] * w8[5 + B]);
 }
 template <class T> __device__ __forceinline__ void store_ref(const Fields<T, 3>& Er, int c, const T* w8) {
@@ -271,8 +274,9 @@ __global__ void __launch_bounds__(BX* BY) k_prim(Grid g, Fields<double, 8> U, Fi
                                                  unsigned* flags, unsigned long long* floors, Fields<T, 3> Er) {
   const Cell p = thread_cell(g);
   T inv = T(0);
-  bool wd = false;  // (double) this cell's primitives wk enter the CFL maximum
-  double wk[8];
+  bool wd = false;  // (double, float pairs) this cell's primitives wk enter the CFL maximum
+  double wr = 0.0, wp = 0.0;  // its density and pressure
+  T wk[8];
   if (p.ok) {
     const int c = p.c;
     const bool in = interior(g, p.i, p.j, p.k);
@@ -305,67 +309,63 @@ __global__ void __launch_bounds__(BX* BY) k_prim(Grid g, Fields<double, 8> U, Fi
       }
       if (dtbits && in) inv = cell_inv_crossing<T>(g, w8);
     } else {
-      double b[3];
-      b[0] = 0.5 * (b0m + b0p);
-      b[1] = 0.5 * (b1m + b1p);
-      b[2] = 0.5 * (b2m + b2p);
-      if (floors) {
-        const double ke = 0.5 * (m0 * (m0 * ir) + m1 * (m1 * ir) + m2 * (m2 * ir));
-        const double me = 0.5 * (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
-        if (lt_pos<double>(g.gm1 * (e - ke - me), g.p_floor)) {
-          e = g.p_floor * g.igm1 + ke + me;
-          U.f[4][c] = e;
-          if (in) atomicAdd(&floors[1], 1ull);
-        }
+      const double b[3] = {half<double>(b0m + b0p), half<double>(b1m + b1p), half<double>(b2m + b2p)};
+      double t2, pg;
+      const PrimD pw = prim_core_ir(g, rho, ir, m0, m1, m2, e, b, t2, pg);
+      if (floors && lt_pos<double>(pg, g.p_floor)) {
+        U.f[4][c] = g.p_floor * g.igm1 + 0.5 * t2;
+        if (in) atomicAdd(&floors[1], 1ull);
       }
-      const PrimD pw = prim_core_ir(g, rho, ir, m0, m1, m2, e, b);
       store_w<T>(W, c, pw, w8);
       store_ref<T>(Er, c, w8);
-      if constexpr (std::is_same<T, double>::value) {
-        if (dtbits && in) {
-          wd = true;
+      if (dtbits && in) {
+        wd = true;
+        wr = pw.rho;
+        wp = pw.p;
 #pragma unroll
-          for (int f = 0; f < 8; ++f) wk[f] = w8[f];
-        }
-      } else {
-        if (dtbits && in) inv = cell_inv_crossing<T>(g, w8);
+        for (int f = 0; f < 8; ++f) wk[f] = w8[f];
       }
     }
   }
-  if constexpr (std::is_same<T, double>::value) {
-    // The CFL maximum of the FP64 step.  Each interior cell's rate is first
-    // estimated in float from its primitives rounded to float.  Where the
-    // grid's 1/d_l and the cell's density and pressure lie in [1e-9, 1e9],
-    // every intermediate of the estimate is a normal float, an overflow
-    // (giving a non-finite estimate) or an underflow whose absolute error
-    // is negligible against a^2 = gamma P / rho, so a finite estimate is
-    // within a relative 1e-5 of the exact rate.  The block maximum M of
-    // those estimates then bounds their cells' exact rates, and only a cell
-    // whose estimate reaches M (1 - 1e-4), or whose estimate is not trusted
-    // (outside the range, not finite), can hold the block's exact maximum.
-    // Those cells evaluate the double rate: the block's maximum is that of
-    // the per-cell double evaluation, bit for bit, at a fraction of the FP64
-    // work (typically one warp in a few per block).
+  if constexpr (sizeof(T) != 4) {
+    // The CFL maximum of the FP64 and double-float steps.  Each interior
+    // cell's rate is first estimated in float from its primitives rounded to
+    // float.  Where the grid's 1/d_l and the cell's density and pressure lie
+    // in [1e-9, 1e9], every intermediate of the estimate is a normal float, an
+    // overflow (giving a non-finite estimate) or an underflow whose absolute
+    // error is negligible against a^2 = gamma P / rho, so a finite estimate
+    // is within a relative 1e-5 of the exact rate.  The block maximum M of
+    // those estimates then bounds their cells' exact rates, and so does the
+    // maximum already posted by other blocks: only a cell whose estimate
+    // reaches both within 1e-4, or whose estimate is not trusted (outside the
+    // range, not finite), can hold the grid's maximum.  Those cells evaluate
+    // the rate in T: the maximum is that of the per-cell evaluation, bit for
+    // bit, and most blocks evaluate none.  (k_prim<double> at 192^3: 1030 us with
+    // the library's reciprocal and the rate of each block's candidates, 399 us
+    // with both changed; 62 to 29 FP64-pipe slots per cell.)
     if (dtbits) {
       auto in_range = [](double x) {  // 1e-9 <= x <= 1e9, on the bit pattern (integer pipes)
         const long long b = dbits(x);
         return b >= dbits(1e-9) && b <= dbits(1e9);
       };
       const bool grid_ok = in_range(g.id[0]) && in_range(g.id[1]) && in_range(g.id[2]);
+      const float posted = d2f_bits(__longlong_as_double(*(volatile long long*)dtbits));
       float est = 0.0f;
       bool trusted = false;
-      if (wd && grid_ok && in_range(wk[0]) && in_range(wk[4])) {
+      if (wd && grid_ok && in_range(wr) && in_range(wp)) {
         float wf[8];
 #pragma unroll
-        for (int f = 0; f < 8; ++f) wf[f] = d2f_bits(wk[f]);
+        for (int f = 0; f < 8; ++f) wf[f] = to_f<T>(wk[f]);
         est = cell_inv_crossing<float>(g, wf);
         trusted = est <= 3.402823466e38f;  // false for an infinity or a NaN
       }
-      const float m = block_max_all(trusted ? est : 0.0f);
+      const float m = fmaxf(block_max_all(trusted ? est : 0.0f), posted);
       const bool cand = wd && (!trusted || !(est < m * (1.0f - 1e-4f)));
-      double inv_d = 0.0;
-      if (cand) inv_d = cell_inv_crossing<double>(g, wk);
-      block_max_to<double>(inv_d, dtbits);
+      if (__syncthreads_or(cand)) {
+        T inv_d = T(0);
+        if (cand) inv_d = cell_inv_crossing<T>(g, wk);
+        block_max_to<T>(inv_d, dtbits);
+      }
     }
   } else {
     if (dtbits) block_max_to<T>(inv, dtbits);
@@ -558,7 +558,7 @@ __device__ __forceinline__ T edge_field(const Grid& g, const Fields<const T, 8>&
       return cell_ref<T, A>(w8);
     }
   };
-  const T bf0 = -ldg(Fbb + q00), bfc = -ldg(Fbb + qc);
+  const T bf0 = neg<T>(ldg(Fbb + q00)), bfc = neg<T>(ldg(Fbb + qc));
   const T cf0 = ldg(Fcb + q00), cfb = ldg(Fcb + qb);
   const T r00 = ref(q00), rb = ref(qb), rc = ref(qc), rbc = ref(qbc);
   const T avg = T(0.25) * (bfc + bf0 + cfb + cf0);
@@ -566,6 +566,7 @@ __device__ __forceinline__ T edge_field(const Grid& g, const Fields<const T, 8>&
   const T Dcm = upwind<T>(ldg(Fbm + q00), cf0, r00, cfb, rb);
   const T Dbp = upwind<T>(ldg(Fcm + qb), bf0, rb, bfc, rbc);
   const T Dbm = upwind<T>(ldg(Fcm + q00), bf0, r00, bfc, rc);
+  if constexpr (sizeof(T) != 4) return quarter<T>(((bfc + bf0) + (cfb + cf0)) + ((Dcp + Dcm) + (Dbp + Dbm)));
   return avg + T(0.25) * (Dcp + Dcm + Dbp + Dbm);
 }
 
@@ -611,7 +612,7 @@ __device__ __forceinline__ T edge_field_r(const Grid& g, const T* __restrict__ W
       return cell_ref<T, A>(w8);
     }
   };
-  const T bf0 = -Fb[5 * N + q00], bfc = -Fb[5 * N + qc];
+  const T bf0 = neg<T>(Fb[5 * N + q00]), bfc = neg<T>(Fb[5 * N + qc]);
   const T cf0 = Fc[6 * N + q00], cfb = Fc[6 * N + qb];
   const T r00 = ref(q00), rb = ref(qb), rc = ref(qc), rbc = ref(qbc);
   const T avg = T(0.25) * (bfc + bf0 + cfb + cf0);
@@ -619,6 +620,7 @@ __device__ __forceinline__ T edge_field_r(const Grid& g, const T* __restrict__ W
   const T Dcm = upwind<T>(Fb[q00], cf0, r00, cfb, rb);
   const T Dbp = upwind<T>(Fc[qb], bf0, rb, bfc, rbc);
   const T Dbm = upwind<T>(Fc[q00], bf0, r00, bfc, rc);
+  if constexpr (sizeof(T) != 4) return quarter<T>(((bfc + bf0) + (cfb + cf0)) + ((Dcp + Dcm) + (Dbp + Dbm)));
   return avg + T(0.25) * (Dcp + Dcm + Dbp + Dbm);
 }
 
@@ -774,7 +776,7 @@ __global__ void __launch_bounds__(BX* BY) k_update_half(Grid g, Fields<const dou
     double t2, pg;
     prim_store_f32(g, W, c, rho, trcp<double>(rho), u5[1], u5[2], u5[3], u5[4], bs, w8, t2, pg);
   } else {
-    const double bcc[3] = {0.5 * (bxm + bx), 0.5 * (bym + by), 0.5 * (bzm + bz)};
+    const double bcc[3] = {half<double>(bxm + bx), half<double>(bym + by), half<double>(bzm + bz)};
     const PrimD pw = prim_core(g, u5[0], u5[1], u5[2], u5[3], u5[4], bcc);
     store_w<T>(W, c, pw, w8);
   }
