@@ -47,6 +47,7 @@ struct mhd_ctx {
   size_t adj_bytes;
   // optional per-stage CUDA-event timing (mhd_profile_enable)
   int prof_on;
+  bool fuse;                    // three-axis launches (WL, WR hold all three axes)
   std::vector<ProfRec> prof;
   std::vector<cudaEvent_t> ev_pool;
   size_t ev_used;
@@ -104,10 +105,11 @@ Layout layout_of(const mhd_config& c) {
   off += up(21 * N * ts);
   L.E = off;
   off += up(3 * N * ts);
+  const size_t faces = mhd::fuse_axes(np[0], np[1], np[2]) ? 21 : 7;
   L.WL = off;
-  off += up(7 * N * ts);
+  off += up(faces * N * ts);
   L.WR = off;
-  off += up(7 * N * ts);
+  off += up(faces * N * ts);
   L.Bh = off;
   off += up(3 * N * ts);
   L.Er = off;
@@ -189,13 +191,20 @@ template <class T> void step_body(mhd_ctx* c, double* U, int recon) {
   T* W = as<T>(c->W);
   T* F = as<T>(c->F);
   T* E = as<T>(c->E);
-  for (int a = 0; a < 3; ++a)  // Steps 2-3
+  const bool fuse = c->fuse;
+  if (fuse) prof(c, MHD_STAGE_FLUX_PCM, [&] { Launch<T>::flux_pcm3(g, W, U, F, s); });
+  for (int a = 0; a < 3 && !fuse; ++a)  // Steps 2-3
     prof(c, MHD_STAGE_FLUX_PCM, [&] { Launch<T>::flux_pcm(g, a, W, U, F, s); });
   T* Er = as<T>(c->Er);
   prof(c, MHD_STAGE_EMF, [&] { Launch<T>::emf(g, W, F, E, s, Er); });        // Step 4
   prof(c, MHD_STAGE_UPDATE_HALF,
        [&] { Launch<T>::update_half(g, U, F, E, c->scal, W, as<T>(c->Bh), c->flags, s, Er); });  // Step 5
-  for (int a = 0; a < 3; ++a) {                                               // Steps 6-7
+  if (fuse) {
+    prof(c, MHD_STAGE_RECON, [&] { Launch<T>::recon3(g, recon, W, as<T>(c->WL), as<T>(c->WR), s); });
+    prof(c, MHD_STAGE_FLUX_HLLD,
+         [&] { Launch<T>::flux_hlld3(g, as<T>(c->WL), as<T>(c->WR), as<T>(c->Bh), F, s); });
+  }
+  for (int a = 0; a < 3 && !fuse; ++a) {                                      // Steps 6-7
     prof(c, MHD_STAGE_RECON, [&] { Launch<T>::recon(g, recon, a, W, as<T>(c->WL), as<T>(c->WR), s); });
     prof(c, MHD_STAGE_FLUX_HLLD,
          [&] { Launch<T>::flux_hlld(g, a, as<T>(c->WL), as<T>(c->WR), as<T>(c->Bh), F, s); });
@@ -463,10 +472,15 @@ int adjoint_step(mhd_ctx* c, const double* Un, double dt, const double* gUp, dou
   double* part1 = cfl ? b.part + b.nparts : nullptr;
   // forward recompute (Steps 1-8; W^n is already in place after the dt reduction)
   if (!cfl) Launch<T>::prim(g, U, b.Wn, nullptr, c->flags, nullptr, s);
-  for (int a = 0; a < 3; ++a) Launch<T>::flux_pcm(g, a, b.Wn, U, b.Fn, s);
+  if (c->fuse) Launch<T>::flux_pcm3(g, b.Wn, U, b.Fn, s);
+  for (int a = 0; a < 3 && !c->fuse; ++a) Launch<T>::flux_pcm(g, a, b.Wn, U, b.Fn, s);
   Launch<T>::emf(g, b.Wn, b.Fn, b.Eh, s);
   mhd::AdjLaunch<T>::fwd_half_keep(g, U, b.Fn, b.Eh, dt, b.Wh, b.Bh, b.Uh, s);
-  for (int a = 0; a < 3; ++a) {
+  if (c->fuse) {
+    Launch<T>::recon3(g, rc, b.Wh, b.WLa, b.WRa, s);
+    Launch<T>::flux_hlld3(g, b.WLa, b.WRa, b.Bh, b.Fh, s);
+  }
+  for (int a = 0; a < 3 && !c->fuse; ++a) {
     Launch<T>::recon(g, rc, a, b.Wh, b.WLa + a * 7 * N, b.WRa + a * 7 * N, s);
     Launch<T>::flux_hlld(g, a, b.WLa + a * 7 * N, b.WRa + a * 7 * N, b.Bh, b.Fh, s);
   }
@@ -623,6 +637,7 @@ int mhd_init(mhd_ctx** out, const mhd_config* cfg, void* stream) {
   }
   c->stream = static_cast<cudaStream_t>(stream);
   c->ts = cfg->precision == MHD_FP32_BULK ? 4 : 8;
+  c->fuse = mhd::fuse_axes(np[0], np[1], np[2]);
   const Layout L = layout_of(*cfg);
   c->ws_bytes = L.total;
   cudaGetLastError();

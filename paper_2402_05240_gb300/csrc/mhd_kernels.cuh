@@ -59,11 +59,11 @@ struct Cell {
   bool ok;
 };
 
-__device__ __forceinline__ Cell thread_cell(const Grid& g) {
+__device__ __forceinline__ Cell thread_cell(const Grid& g, int k) {
   Cell p;
   p.i = blockIdx.x * BX + threadIdx.x;
   p.j = blockIdx.y * BY + threadIdx.y;
-  p.k = blockIdx.z;
+  p.k = k;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nxy = nx * ny;
   p.ok = p.i < nx && p.j < ny;
   p.c = (p.k * ny + p.j) * nx + p.i;
@@ -74,6 +74,18 @@ __device__ __forceinline__ Cell thread_cell(const Grid& g) {
   p.m[2] = p.k == 0 ? (nz - 1) * nxy : -nxy;
   p.p[2] = p.k == nz - 1 ? (1 - nz) * nxy : nxy;
   return p;
+}
+
+__device__ __forceinline__ Cell thread_cell(const Grid& g) { return thread_cell(g, blockIdx.z); }
+
+// Launches over the three axes at once (small grids): grid z runs over the
+// axes' planes, axis by axis.
+__device__ __forceinline__ int block_axis(const Grid& g) {
+  return (int)blockIdx.z < g.n[2] ? 0 : ((int)blockIdx.z < 2 * g.n[2] ? 1 : 2);
+}
+inline dim3 grid3_of(const Grid& g) {
+  const dim3 d = grid_of(g);
+  return dim3(d.x, d.y, 3 * d.z);
 }
 
 // offset from cell p to p + s e_A (periodic), |s| < n[A]
@@ -399,17 +411,33 @@ template <int A, class T> __device__ __forceinline__ void load_dir(const Fields<
 // holds too many registers for the occupancy the double-float arithmetic
 // needs to hide its latencies.  BA: the face field B_A of the state.
 template <class T, int A>
-__global__ void __launch_bounds__(BX* BY) k_flux_pcm(Grid g, Fields<const T, 8> W, const double* __restrict__ BA,
-                                                     Fields<T, 7> FA) {
-  const Cell p = thread_cell(g);
-  if (!p.ok) return;
+__device__ __forceinline__ void flux_pcm_cell(const Grid& g, const Cell& p, const Fields<const T, 8>& W,
+                                              const double* BA, T* const* FA) {
   const int c = p.c;
   T wl[7], wr[7], f[7];
   load_dir<A>(W, c, wl);
   load_dir<A>(W, c + p.p[A], wr);
   hlld<T>(from_d<T>(g.gamma), from_d<T>(g.igm1), wl, wr, from_d<T>(ldg(BA + c)), f);
 #pragma unroll
-  for (int q = 0; q < 7; ++q) FA.f[q][c] = f[q];
+  for (int q = 0; q < 7; ++q) FA[q][c] = f[q];
+}
+
+template <class T, int A>
+__global__ void __launch_bounds__(BX* BY) k_flux_pcm(Grid g, Fields<const T, 8> W, const double* __restrict__ BA,
+                                                     Fields<T, 7> FA) {
+  const Cell p = thread_cell(g);
+  if (p.ok) flux_pcm_cell<T, A>(g, p, W, BA, FA.f);
+}
+
+template <class T>
+__global__ void __launch_bounds__(BX* BY) k_flux_pcm3(Grid g, Fields<const T, 8> W, Fields<const double, 3> B,
+                                                      Fields<T, 21> F) {
+  const int a = block_axis(g);
+  const Cell p = thread_cell(g, blockIdx.z - a * g.n[2]);
+  if (!p.ok) return;
+  if (a == 0) flux_pcm_cell<T, 0>(g, p, W, B.f[0], F.f);
+  else if (a == 1) flux_pcm_cell<T, 1>(g, p, W, B.f[1], F.f + 7);
+  else flux_pcm_cell<T, 2>(g, p, W, B.f[2], F.f + 14);
 }
 
 // ------------------------------------------------------------------ Step 6 --
@@ -469,23 +497,61 @@ __global__ void __launch_bounds__(BX* BY, ReconMinBlocks<T, RECON>::v) k_recon(G
   }
 }
 
+template <class T, int RECON, int A>
+__device__ __forceinline__ void recon_axis(const Grid& g, const Fields<const T, 8>& W, const Cell& p,
+                                           const Fields<T, 21>& WL, const Fields<T, 21>& WR) {
+  T wl[7], wr[7];
+  recon_cell<T, RECON, A>(g, W, p, wl, wr);
+#pragma unroll
+  for (int q = 0; q < 7; ++q) {
+    WL.f[A * 7 + q][p.c] = wl[q];
+    WR.f[A * 7 + q][p.c] = wr[q];
+  }
+}
+template <class T, int RECON>
+__global__ void __launch_bounds__(BX* BY, ReconMinBlocks<T, RECON>::v) k_recon3(Grid g, Fields<const T, 8> W,
+                                                                              Fields<T, 21> WL, Fields<T, 21> WR) {
+  const int a = block_axis(g);
+  const Cell p = thread_cell(g, blockIdx.z - a * g.n[2]);
+  if (!p.ok) return;
+  if (a == 0) recon_axis<T, RECON, 0>(g, W, p, WL, WR);
+  else if (a == 1) recon_axis<T, RECON, 1>(g, W, p, WL, WR);
+  else recon_axis<T, RECON, 2>(g, W, p, WL, WR);
+}
+
 // ------------------------------------------------------------------ Step 7 --
 // BfA: the half-step face field B_A
 template <class T, int A>
-__global__ void __launch_bounds__(BX* BY) k_flux_hlld(Grid g, Fields<const T, 7> WL, Fields<const T, 7> WR,
-                                                      const T* __restrict__ BfA, Fields<T, 7> FA) {
-  const Cell p = thread_cell(g);
-  if (!p.ok) return;
+__device__ __forceinline__ void flux_hlld_cell(const Grid& g, const Cell& p, const T* const* WL, const T* const* WR,
+                                               const T* BfA, T* const* FA) {
   const int c = p.c, cn = c + p.p[A];
   T wl[7], wr[7], f[7];
 #pragma unroll
   for (int q = 0; q < 7; ++q) {
-    wl[q] = ldg(WL.f[q] + c);
-    wr[q] = ldg(WR.f[q] + cn);
+    wl[q] = ldg(WL[q] + c);
+    wr[q] = ldg(WR[q] + cn);
   }
   hlld<T>(from_d<T>(g.gamma), from_d<T>(g.igm1), wl, wr, ldg(BfA + c), f);
 #pragma unroll
-  for (int q = 0; q < 7; ++q) FA.f[q][c] = f[q];
+  for (int q = 0; q < 7; ++q) FA[q][c] = f[q];
+}
+
+template <class T, int A>
+__global__ void __launch_bounds__(BX* BY) k_flux_hlld(Grid g, Fields<const T, 7> WL, Fields<const T, 7> WR,
+                                                      const T* __restrict__ BfA, Fields<T, 7> FA) {
+  const Cell p = thread_cell(g);
+  if (p.ok) flux_hlld_cell<T, A>(g, p, WL.f, WR.f, BfA, FA.f);
+}
+
+template <class T>
+__global__ void __launch_bounds__(BX* BY) k_flux_hlld3(Grid g, Fields<const T, 21> WL, Fields<const T, 21> WR,
+                                                       Fields<const T, 3> Bf, Fields<T, 21> F) {
+  const int a = block_axis(g);
+  const Cell p = thread_cell(g, blockIdx.z - a * g.n[2]);
+  if (!p.ok) return;
+  if (a == 0) flux_hlld_cell<T, 0>(g, p, WL.f, WR.f, Bf.f[0], F.f);
+  else if (a == 1) flux_hlld_cell<T, 1>(g, p, WL.f + 7, WR.f + 7, Bf.f[1], F.f + 7);
+  else flux_hlld_cell<T, 2>(g, p, WL.f + 14, WR.f + 14, Bf.f[2], F.f + 14);
 }
 
 // The float Riemann kernel keeps restrict-qualified base pointers with
@@ -1073,6 +1139,26 @@ void Launch<T>::recon(const Grid& g, int rc, int a, const T* W, T* WL, T* WR, cu
   else if (rc == 1) launch_recon<T, 1>(g, a, Wf, L, R, s);
   else if (rc == 2) launch_recon<T, 2>(g, a, Wf, L, R, s);
   else launch_recon<T, 3>(g, a, Wf, L, R, s);
+}
+template <class T>
+void Launch<T>::flux_pcm3(const Grid& g, const T* W, const double* U, T* F, cudaStream_t s) {
+  k_flux_pcm3<T><<<grid3_of(g), dim3(BX, BY), 0, s>>>(g, fields<8>(W, g.N), fields<3>(U + 5 * g.N, g.N),
+                                                      fields<21>(F, g.N));
+}
+template <class T>
+void Launch<T>::recon3(const Grid& g, int rc, const T* W, T* WL, T* WR, cudaStream_t s) {
+  const Fields<const T, 8> Wf = fields<8>(W, g.N);
+  const Fields<T, 21> L = fields<21>(WL, g.N), R = fields<21>(WR, g.N);
+  const dim3 gr = grid3_of(g), bl(BX, BY);
+  if (rc == 0) k_recon3<T, 0><<<gr, bl, 0, s>>>(g, Wf, L, R);
+  else if (rc == 1) k_recon3<T, 1><<<gr, bl, 0, s>>>(g, Wf, L, R);
+  else if (rc == 2) k_recon3<T, 2><<<gr, bl, 0, s>>>(g, Wf, L, R);
+  else k_recon3<T, 3><<<gr, bl, 0, s>>>(g, Wf, L, R);
+}
+template <class T>
+void Launch<T>::flux_hlld3(const Grid& g, const T* WL, const T* WR, const T* Bf, T* F, cudaStream_t s) {
+  k_flux_hlld3<T><<<grid3_of(g), dim3(BX, BY), 0, s>>>(g, fields<21>(WL, g.N), fields<21>(WR, g.N),
+                                                       fields<3>(Bf, g.N), fields<21>(F, g.N));
 }
 template <class T>
 void Launch<T>::flux_hlld(const Grid& g, int a, const T* WL, const T* WR, const T* Bf, T* F, cudaStream_t s) {

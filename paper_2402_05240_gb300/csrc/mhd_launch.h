@@ -13,6 +13,20 @@ inline long long cell_blocks(int nx, int ny, int nz) {
   return (long long)((nx + BX - 1) / BX) * ((ny + BY - 1) / BY) * nz;
 }
 
+// Grids of up to kFuseBlocks thread blocks per axis run each three-axis stage
+// (predictor fluxes, reconstruction, corrector fluxes) as one launch of three
+// times the blocks: 9 launches per step instead of 15, and three times the
+// blocks to fill the SMs with.  It needs the interface states of all axes at
+// once (28 more words per cell).  Measured per PPMC step, three launches /
+// one, at 16^3, 32^3, 64^3, 96^3, 128^3, 160^3: FP32-bulk 75 / 47, 78 / 55,
+// 170 / 143, 415 / 388, 857 / 834, 1562 / 1551 us; FP64 182 / 113, 266 / 238,
+// 1419 / 1355, 4352 / 4276, 9957 / 9877, 19085 / 19005 us.  The line is at
+// 128^3, where the gain falls below 3 % and the words pass 0.5 GB.
+constexpr long long kFuseBlocks = 16384;
+inline bool fuse_axes(int nx, int ny, int nz) {
+  return cell_blocks(nx, ny, nz) <= kFuseBlocks && nz <= 65535 / 3;
+}
+
 struct Grid {
   int n[3];          // nx, ny, nz
   long long N;       // nx * ny * nz
@@ -57,6 +71,11 @@ template <class T> struct Launch {
   static void flux_pcm(const Grid& g, int a, const T* W, const double* U, T* F, cudaStream_t s);  // axis a
   static void recon(const Grid& g, int rc, int a, const T* W, T* WL, T* WR, cudaStream_t s);
   static void flux_hlld(const Grid& g, int a, const T* WL, const T* WR, const T* Bf, T* F, cudaStream_t s);
+  // the same over all three axes in one launch (small grids: fuse_axes);
+  // WL, WR hold 21 fields, axis by axis
+  static void flux_pcm3(const Grid& g, const T* W, const double* U, T* F, cudaStream_t s);
+  static void recon3(const Grid& g, int rc, const T* W, T* WL, T* WR, cudaStream_t s);
+  static void flux_hlld3(const Grid& g, const T* WL, const T* WR, const T* Bf, T* F, cudaStream_t s);
   // Er: the reference fields written with W (null: formed from W)
   static void emf(const Grid& g, const T* W, const T* F, T* E, cudaStream_t s, const T* Er = nullptr);
   static void update_half(const Grid& g, const double* U, const T* F, const T* E, const double* dtp, T* W, T* Bh,
