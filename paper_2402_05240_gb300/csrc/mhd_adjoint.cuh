@@ -884,13 +884,332 @@ __device__ __forceinline__ void phys_cons_vjp(T gm1i, const T* w, T bn, const T*
   gw[6] += gbz;
 }
 
+// Reverse of hlld_diff (double and float pairs): the same increments, so about
+// 200 operations after the forward's 90 to 132, against about 850 for the
+// reverse of the jump form, which carries both sides' star states and three
+// conserved vectors.  Measured: FP64 PPMC adjoint step at 128^3 55.7 -> 48.0 ms,
+// double-float rollout at 64^3 14.3 -> 10.8 ms (1 KB of register spill per
+// thread down to 0.1 KB).  The mass flux's rounding switch (rs == r) carries no
+// derivative of its own.
+template <class T>
+__device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, const T* wr, T bn, const T* gf, T* gwl,
+                                              T* gwr, T& gbn) {
+  // forward (hlld_diff)
+  const T bn2 = bn * bn;
+  const T btL = wl[5] * wl[5] + wl[6] * wl[6], btR = wr[5] * wr[5] + wr[6] * wr[6];
+  const T bbL = bn2 + btL, bbR = bn2 + btR;
+  const T ptL = wl[4] + half<T>(bbL), ptR = wr[4] + half<T>(bbR);
+  auto root = [&](T p, T bb, T bt) -> T {
+    const T gp = gamma * p;
+    const T dd = gp - bb;
+    return tsqrt<T>(dd * dd + quad<T>(gp) * bt);
+  };
+  const T sL = root(wl[4], bbL, btL), sR = root(wr[4], bbR, btR);
+  const T XL = gamma * wl[4] + bbL + sL, XR = gamma * wr[4] + bbR + sR;
+  const bool lmax = !nonneg_lt<T>(XL * wr[0], XR * wl[0]);
+  const T irc = trcp<T>(lmax ? wl[0] : wr[0]);
+  const T c2 = half<T>(lmax ? XL : XR) * irc;
+  const T cmax = tsqrt<T>(c2);
+  const T SL = min_s<T>(wl[1], wr[1]) - cmax;
+  const T SR = max_s<T>(wl[1], wr[1]) + cmax;
+  const bool sub = !ge0<T>(SL) && !le0<T>(SR);
+  T rdL = T(0), rdR = T(0), dlL = T(0), dlR = T(0), SM = T(0), pts = T(0), iden = T(0);
+  if (sub) {
+    rdL = wl[0] * (SL - wl[1]);
+    rdR = wr[0] * (SR - wr[1]);
+    iden = trcp<T>(rdR - rdL);
+    const T du = wr[1] - wl[1], dp = ptL - ptR;
+    dlL = (rdR * du + dp) * iden;
+    dlR = (rdL * du + dp) * iden;
+    SM = wl[1] + dlL;
+    pts = ptL + rdL * dlL;
+  }
+  const bool left = sub ? ge0<T>(SM) : ge0<T>(SL);
+  const T* w = left ? wl : wr;
+  const T* wo = left ? wr : wl;
+  const T r = w[0], u = w[1], v = w[2], vw = w[3], by = w[5], bz = w[6];
+  const T bt = left ? btL : btR, v2 = u * u + v * v + vw * vw;
+  const T hb = half<T>(left ? bbL : bbR), pt = left ? ptL : ptR;
+  const T e = w[4] * gm1i + (half<T>(r) * v2 + hb);
+  const T mu = r * u;
+  const T vby = v * by + vw * bz;
+
+  // reverse of the physical flux of the selected side, and the cotangents of
+  // the increments m1, C, A, dE
+  T m1 = T(0), C = bn, A = u, S = T(0);
+  T rs = T(0), z = T(0), rd = T(0), dl = T(0), t = T(0), rz = T(0), Sd = T(0), iSd = T(0), iD = T(0), rsq = T(0);
+  T Ss = T(0);
+  bool inner = false;
+  if (sub) {
+    S = left ? SL : SR;
+    dl = left ? dlL : dlR;
+    rd = left ? rdL : rdR;
+    Sd = S - SM;
+    iSd = trcp<T>(Sd);
+    rs = rd * iSd;
+    const T D = rd * Sd - bn2;
+    if (!abs_lt<T>(D, Eps<T>::hlld * pts)) {
+      iD = trcp<T>(D);
+      z = dl * iD;
+    }
+    t = bn * z;
+    rz = rd * z;
+    m1 = S * (r * (dl * iSd));
+    C = bn + S * rs * t;
+    A = u + S * rz;
+    rsq = trsqrt<T>(rs);
+    const T cA = fabs(bn) * rsq;
+    Ss = left ? SM - cA : SM + cA;
+    inner = (left ? lt0<T>(Ss) : ge0<T>(Ss)) && !nonneg_lt<T>(half<T>(bn2), Eps<T>::hlld * pts);
+  }
+  const T f0 = mu + m1;
+  const T gf0 = gf[0] + gf[2] * v + gf[3] * vw;
+  const T gmu = gf0 + gf[1] * u;
+  T g_r = gmu * u;
+  T g_u = gmu * r + gf[1] * mu + gf[4] * (e + pt - bn2);
+  T g_v = gf[2] * f0 - gf[5] * bn, g_vw = gf[3] * f0 - gf[6] * bn;
+  T g_by = gf[5] * A - gf[2] * C, g_bz = gf[6] * A - gf[3] * C;
+  T g_vby = -(gf[4] * bn);
+  T g_bn = -(gf[5] * v + gf[6] * vw + gf[4] * (twice<T>(u * bn) + vby) + twice<T>(gf[1] * bn));
+  const T gC = -(gf[2] * by + gf[3] * bz), gA = gf[5] * by + gf[6] * bz;
+  T g_e = gf[4] * u, g_pt = gf[1] + g_e;
+  g_bn += gC;
+  g_u += gA;
+  // cotangents of the other side's state (u, B_t, v, w through its star state)
+  // and of both sides' rd, dl, S
+  T go2 = T(0), go3 = T(0), go5 = T(0), go6 = T(0);
+  T g_rd = T(0), g_dl = T(0), g_S = T(0), g_SM = T(0), g_bt = T(0);
+  T g_rdo = T(0), g_dlo = T(0), g_So = T(0);
+  if (sub) {
+    T g_rs = T(0), g_t = T(0), g_rz = T(0), g_iSd = T(0);
+    if (inner) {
+      const T rdo = left ? rdR : rdL, dlo = left ? dlR : dlL;
+      const T Sdo = (left ? SR : SL) - SM;
+      const T iSdo = trcp<T>(Sdo);
+      const T rso = rdo * iSdo;
+      const T Do = rdo * Sdo - bn2;
+      T iDo = T(0);
+      if (!abs_lt<T>(Do, Eps<T>::hlld * pts)) iDo = trcp<T>(Do);
+      const T zo = dlo * iDo;
+      const T q = T(1) + rz, to = bn * zo, qo = T(1) + rdo * zo;
+      const T vs = v - by * t, ws = vw - bz * t, bys = by * q, bzs = bz * q;
+      const T vo = wo[2] - wo[5] * to, wwo = wo[3] - wo[6] * to;
+      const T rsqo = trsqrt<T>(rso);
+      const T sq = rs * rsq, sqo = rso * rsqo;
+      const T inv = trcp<T>(sq + sqo);
+      const T sg = (gt0<T>(bn) == left) ? T(1) : T(-1);
+      const T dv = vo - vs, dw = wwo - ws;
+      const T Dy = (times_sign<T>(wo[5] * qo - bys, sg) + sqo * dv) * inv;
+      const T Dz = (times_sign<T>(wo[6] * qo - bzs, sg) + sqo * dw) * inv;
+      const T gg = times_sign<T>(sq, sg);
+      const T ay = Ss * Dy, az = Ss * Dz;
+      const T vd = vs + Dy, wd = ws + Dz;
+      const T Py = bys + gg * vd, Pz = bzs + gg * wd;
+      // reverse
+      g_rs += gf[2] * ay + gf[3] * az;
+      const T g4g = gf[4] * gg;
+      const T g_ay = gf[2] * rs + g4g * Py + gf[5] * gg, g_az = gf[3] * rs + g4g * Pz + gf[6] * gg;
+      const T gPy = g4g * ay, gPz = g4g * az;
+      const T g_gg = gf[4] * (ay * Py + az * Pz) + gf[5] * ay + gf[6] * az + (gPy * vd + gPz * wd);
+      T g_vs = gPy * gg, g_ws = gPz * gg;
+      const T g_Dy = g_vs + g_ay * Ss, g_Dz = g_ws + g_az * Ss;
+      const T g_Ss = g_ay * Dy + g_az * Dz;
+      const T ny = g_Dy * inv, nz = g_Dz * inv;
+      const T g_sum = -(ny * Dy + nz * Dz);
+      const T hy = times_sign<T>(ny, sg), hz = times_sign<T>(nz, sg);
+      const T g_bys = gPy - hy, g_bzs = gPz - hz;
+      const T g_vo = ny * sqo, g_wwo = nz * sqo;
+      g_vs -= g_vo;
+      g_ws -= g_wwo;
+      const T g_sqo = g_sum + (ny * dv + nz * dw);
+      T g_sq = g_sum + times_sign<T>(g_gg, sg);
+      // Ss = S_M -+ |bn| / sq
+      g_SM += g_Ss;
+      const T gr = g_Ss * rsq;
+      const T sb = gt0<T>(bn) == left ? T(-1) : T(1);
+      g_bn += times_sign<T>(gr, sb);
+      const T ga = gr * (fabs(bn) * rsq);
+      g_sq = left ? T(g_sq + ga) : T(g_sq - ga);
+      g_rs += half<T>(g_sq) * rsq;
+      const T g_rso = half<T>(g_sqo) * rsqo;
+      // star state of the selected side
+      g_v += g_vs;
+      g_vw += g_ws;
+      g_by += g_bys * q - g_vs * t;
+      g_bz += g_bzs * q - g_ws * t;
+      g_t -= g_vs * by + g_ws * bz;
+      g_rz += g_bys * by + g_bzs * bz;
+      // and of the other one
+      const T g_byo = hy, g_bzo = hz;
+      go2 = g_vo;
+      go3 = g_wwo;
+      go5 = g_byo * qo - g_vo * to;
+      go6 = g_bzo * qo - g_wwo * to;
+      const T g_to = -(g_vo * wo[5] + g_wwo * wo[6]);
+      const T g_qo = g_byo * wo[5] + g_bzo * wo[6];
+      g_bn += g_to * zo;
+      const T g_zo = g_to * bn + g_qo * rdo;
+      g_dlo = g_zo * iDo;
+      const T g_Do = -(g_zo * zo * iDo);
+      g_rdo = g_qo * zo + g_Do * Sdo + g_rso * iSdo;
+      g_So = g_Do * rdo - g_rso * rso * iSdo;
+      g_SM -= g_So;
+      g_bn -= twice<T>(bn * g_Do);
+    }
+    // dE = S K iSd, K = (e + p* + u rd) dl - bn dvb
+    const T bbt = bt * t;
+    const T dvb = rz * (vby - bbt) + (bn * dl - bbt);
+    const T H = e + (pt + rd * dl) + u * rd;
+    const T K = H * dl - bn * dvb;
+    const T gE = gf[4];
+    const T gES = gE * S;
+    g_S += gE * (K * iSd);
+    g_iSd += gES * K;
+    const T gK = gES * iSd;
+    g_dl += gK * H;
+    const T gH = gK * dl;
+    g_e += gH;
+    g_pt += gH;
+    g_u += gH * rd;
+    g_rd += gH * (u + dl);
+    g_dl += gH * rd;
+    const T gdvb = -(gK * bn);
+    g_bn += gdvb * dl - gK * dvb;
+    g_dl += gdvb * bn;
+    g_vby += gdvb * rz;
+    g_rz += gdvb * (vby - bbt);
+    const T gbbt = -(gdvb * (T(1) + rz));
+    g_bt += gbbt * t;
+    g_t += gbbt * bt;
+    // A = u + S rz, C = bn + S rs t
+    g_S += gA * rz;
+    g_rz += gA * S;
+    const T gCS = gC * S;
+    g_S += gC * (rs * t);
+    g_rs += gCS * t;
+    g_t += gCS * rs;
+    // m1 = S r dl iSd, entering f0 (gf0) and, times S, f1
+    const T g_m1 = gf0 + gf[1] * S;
+    const T h = dl * iSd, gh = g_m1 * S;
+    g_S += g_m1 * (r * h) + gf[1] * m1;
+    g_r += gh * h;
+    const T ghr = gh * r;
+    g_dl += ghr * iSd;
+    g_iSd += ghr * dl;
+    // rz = rd z, t = bn z, z = dl / D, D = rd Sd - bn2, rs = rd iSd
+    g_rd += g_rz * z;
+    g_bn += g_t * z;
+    const T g_z = g_rz * rd + g_t * bn;
+    g_dl += g_z * iD;
+    const T g_D = -(g_z * z * iD);
+    g_rd += g_D * Sd + g_rs * iSd;
+    g_iSd += g_rs * rd;
+    const T g_Sd = g_D * rd - g_iSd * iSd * iSd;
+    g_bn -= twice<T>(bn * g_D);
+    g_S += g_Sd;
+    g_SM -= g_Sd;
+  }
+  g_v += g_vby * by;
+  g_by += g_vby * v;
+  g_vw += g_vby * bz;
+  g_bz += g_vby * vw;
+  // e = p gm1i + r v^2 / 2 + bb / 2, pt = p + bb / 2, bb = bn2 + bt
+  T g_p = g_e * gm1i + g_pt;
+  const T ger = g_e * r;
+  g_r += half<T>(g_e * v2);
+  g_u += ger * u;
+  g_v += ger * v;
+  g_vw += ger * vw;
+  T g_bb = half<T>(g_e + g_pt);
+  T g_po = T(0), g_ro = T(0), g_uo = T(0), g_bbo = T(0);
+  if (sub) {
+    // middle wave: dl_L = (rd_R du + dp) iden, dl_R = (rd_L du + dp) iden, S_M = u_L + dl_L
+    T g_dlL = left ? g_dl : g_dlo, g_dlR = left ? g_dlo : g_dl;
+    g_dlL += g_SM;
+    const T nL = g_dlL * iden, nR = g_dlR * iden;
+    const T g_den = -(nL * dlL + nR * dlR);
+    const T du = wr[1] - wl[1];
+    T g_rdL = left ? g_rd : g_rdo, g_rdR = left ? g_rdo : g_rd;
+    g_rdR += nL * du + g_den;
+    g_rdL += nR * du - g_den;
+    const T g_du = nL * rdR + nR * rdL, g_dp = nL + nR;
+    // rd = rho (S - u)
+    const T aL = g_rdL * wl[0], aR = g_rdR * wr[0];
+    const T g_uL = g_SM - g_du - aL, g_uR = g_du - aR;
+    const T g_rL = g_rdL * (SL - wl[1]), g_rR = g_rdR * (SR - wr[1]);
+    T g_SL = left ? g_S : g_So, g_SR = left ? g_So : g_S;
+    g_SL += aL;
+    g_SR += aR;
+    g_r += left ? g_rL : g_rR;
+    g_u += left ? g_uL : g_uR;
+    g_ro = left ? g_rR : g_rL;
+    g_uo = left ? g_uR : g_uL;
+    const T hdp = half<T>(g_dp);  // dp = p_L - p_R + (bb_L - bb_R) / 2
+    g_p = left ? T(g_p + g_dp) : T(g_p - g_dp);
+    g_bb = left ? T(g_bb + hdp) : T(g_bb - hdp);
+    g_po = left ? T(-g_dp) : g_dp;
+    g_bbo = left ? T(-hdp) : hdp;
+    // outer speeds: SL = min(uL, uR) - cmax, SR = max(uL, uR) + cmax
+    const T g_c = g_SR - g_SL;
+    const bool lo = wl[1] <= wr[1], hi = wl[1] >= wr[1];  // the left side gives the minimum, the maximum
+    g_u += (left == lo ? g_SL : T(0)) + (left == hi ? g_SR : T(0));
+    g_uo += (left == lo ? T(0) : g_SL) + (left == hi ? T(0) : g_SR);
+    // cmax^2 = X / (2 rho), X = gamma P + bb + s, s = sqrt((gamma P - bb)^2 + 4 gamma P bt)
+    if (gt0<T>(cmax)) {
+      const T g_c2 = half<T>(g_c) * trcp<T>(cmax);
+      const T g_hX = g_c2 * irc;  // of X / 2
+      const T gg = half<T>(g_hX);
+      const T gp = gamma * (lmax ? wl[4] : wr[4]), bbm = lmax ? bbL : bbR, btm = lmax ? btL : btR, sm = lmax ? sL : sR;
+      T g_gp = gg, g_bbm = gg, g_btm = T(0);
+      if (gt0<T>(sm)) {
+        const T is = gg * trcp<T>(sm);
+        const T dd = gp - bbm;
+        g_gp += is * (dd + twice<T>(btm));
+        g_bbm -= is * dd;
+        g_btm = twice<T>(is * gp);
+      }
+      const T g_rm = -(g_hX * c2), g_pm = gamma * g_gp;
+      const bool own = lmax == left;
+      g_r += own ? g_rm : T(0);
+      g_ro += own ? T(0) : g_rm;
+      g_p += own ? g_pm : T(0);
+      g_po += own ? T(0) : g_pm;
+      g_bb += own ? g_bbm : T(0);
+      g_bbo += own ? T(0) : g_bbm;
+      const T two = twice<T>(g_btm);
+      g_bt += own ? g_btm : T(0);
+      go5 += own ? T(0) : T(two * wo[5]);
+      go6 += own ? T(0) : T(two * wo[6]);
+    }
+    const T two = twice<T>(g_bbo);
+    go5 += two * wo[5];
+    go6 += two * wo[6];
+  }
+  g_bn += twice<T>(bn * (g_bb + g_bbo));
+  const T two = twice<T>(g_bt + g_bb);
+  g_by += two * by;
+  g_bz += two * bz;
+  const T gsel[7] = {g_r, g_u, g_v, g_vw, g_p, g_by, g_bz};
+  const T goth[7] = {g_ro, g_uo, go2, go3, g_po, go5, go6};
+#pragma unroll
+  for (int q = 0; q < 7; ++q) {
+    gwl[q] += left ? gsel[q] : goth[q];
+    gwr[q] += left ? goth[q] : gsel[q];
+  }
+  gbn += g_bn;
+}
+
 // Reverse of hlld(): gf = cotangent of the 7 flux components; accumulates
 // gwl[7], gwr[7] and gbn.  Follows the region selection, the degenerate
 // switches and the outer-speed selections of the forward solver.
 template <class T>
 __device__ void hlld_vjp(T gamma, const T* wl, const T* wr, T bn, const T* gf, T* gwl, T* gwr, T& gbn) {
-  const T bn2 = bn * bn;
   const T gm1i = trcp<T>(gamma - T(1));
+  if constexpr (sizeof(T) != 4) {
+    hlld_diff_vjp<T>(gamma, gm1i, wl, wr, bn, gf, gwl, gwr, gbn);
+    return;
+  }
+  const T bn2 = bn * bn;
   T eL, eR, ptL, ptR;
   {
     T bb = bn2 + wl[5] * wl[5] + wl[6] * wl[6];
