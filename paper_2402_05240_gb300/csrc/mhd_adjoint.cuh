@@ -44,7 +44,70 @@ template <class T> struct EigG {
   }
 };
 
-// reverse of eig_left (q = L dw): accumulates gdw and gE
+// Double and float pairs reverse the projections in the coefficient form of
+// eig_left: the projections of a reconstruction accumulate the cotangents of
+// its shared coefficients (fast and slow amplitudes of dP, dB, du; the
+// Alfven ones of dB), and eig_coef_vjp carries them to the eigensystem once:
+// 45 operations per projection against about 95.  With the limiter's reverse
+// (ppm_one_vjp_wide): FP64 PPMC adjoint step at 128^3 48.0 -> 38.0 ms.
+template <class T> struct EigCoefG {
+  T fp, sp, fb, sb, fu, su, z1, z2;
+  __device__ void zero() { fp = sp = fb = sb = fu = su = z1 = z2 = T(0); }
+};
+template <class T>
+__device__ __forceinline__ void eig_left_vjp_wide(const Eig<T>& E, const T* dw, const T* gq, T* gdw, EigG<T>& gE,
+                                                  EigCoefG<T>& gC) {
+  const T n = half<T>(E.ia2);
+  const T naf = n * E.af, nas = n * E.as, ai = E.a * E.isr;
+  const T fp = naf * E.ir, sp = nas * E.ir, fb = nas * ai, sb = naf * ai, fu = naf * E.cf, su = nas * E.cs;
+  const T z = half<T>(times_sign<T>(E.isr, E.sg));
+  const T z1 = E.b1 * z, z2 = E.b2 * z;
+  const T bv = times_sign<T>(E.b1 * dw[2] + E.b2 * dw[3], E.sg);
+  const T bb = E.b1 * dw[5] + E.b2 * dw[6];
+  const T gXf = gq[0] + gq[6], gYf = gq[0] - gq[6];
+  const T gXs = gq[2] + gq[4], gYs = gq[4] - gq[2];
+  const T hZ = half<T>(gq[1] + gq[5]), gZb = gq[1] - gq[5];
+  gC.fp += gXf * dw[4];
+  gC.sp += gXs * dw[4];
+  gC.fb += gXf * bb;
+  gC.sb -= gXs * bb;
+  gC.su += gYf * bv + gYs * dw[1];
+  gC.fu += gYs * bv - gYf * dw[1];
+  gC.z1 += gZb * dw[6];
+  gC.z2 -= gZb * dw[5];
+  const T gbb = gXf * fb - gXs * sb;
+  const T gbv = times_sign<T>(gYf * su + gYs * fu, E.sg);
+  gE.ia2 -= gq[3] * dw[4];
+  gE.b1 += gbv * dw[2] + gbb * dw[5] + hZ * dw[3];
+  gE.b2 += gbv * dw[3] + gbb * dw[6] - hZ * dw[2];
+  gdw[0] = gq[3];
+  gdw[1] = gYs * su - gYf * fu;
+  gdw[2] = gbv * E.b1 - hZ * E.b2;
+  gdw[3] = gbv * E.b2 + hZ * E.b1;
+  gdw[4] = gXf * fp + gXs * sp - gq[3] * E.ia2;
+  gdw[5] = gbb * E.b1 - gZb * z2;
+  gdw[6] = gbb * E.b2 + gZb * z1;
+}
+template <class T> __device__ __forceinline__ void eig_coef_vjp(const Eig<T>& E, const EigCoefG<T>& gC, EigG<T>& gE) {
+  if constexpr (sizeof(T) == 4) return;
+  const T n = half<T>(E.ia2);
+  const T naf = n * E.af, nas = n * E.as, ai = E.a * E.isr;
+  const T gnaf = gC.fp * E.ir + gC.sb * ai + gC.fu * E.cf, gnas = gC.sp * E.ir + gC.fb * ai + gC.su * E.cs;
+  const T gai = gC.fb * nas + gC.sb * naf;
+  gE.ir += gC.fp * naf + gC.sp * nas;
+  gE.cf += gC.fu * naf;
+  gE.cs += gC.su * nas;
+  gE.af += gnaf * n;
+  gE.as += gnas * n;
+  gE.ia2 += half<T>(gnaf * E.af + gnas * E.as);
+  gE.a += gai * E.isr;
+  gE.isr += gai * E.a + times_sign<T>(half<T>(gC.z1 * E.b1 + gC.z2 * E.b2), E.sg);
+  const T z = half<T>(times_sign<T>(E.isr, E.sg));
+  gE.b1 += gC.z1 * z;
+  gE.b2 += gC.z2 * z;
+}
+
+// reverse of eig_left (q = L dw), float: accumulates gdw and gE
 template <class T>
 __device__ __forceinline__ void eig_left_vjp(const Eig<T>& E, T ir, const T* dw, const T* gq, T* gdw, EigG<T>& gE) {
   const T n = T(0.5) * E.ia2;
@@ -125,13 +188,13 @@ __device__ __forceinline__ void eig_right_vjp(const Eig<T>& E, const T* q, const
   const T K = E.af * fp + E.as * sp;
   const T M = E.Qs * fm - E.Qf * sm;
   const T ms = E.As * fp - E.Af * sp;
-  const T ssr = E.sg * E.sr * am;
+  const T ssr = times_sign<T>(E.sr, E.sg) * am;
   gE.b1 += gdw[5] * ms + gdw[6] * ssr + gdw[2] * M + gdw[3] * ap;
   gE.b2 += gdw[6] * ms - gdw[5] * ssr + gdw[3] * M - gdw[2] * ap;
   const T gms = gdw[5] * E.b1 + gdw[6] * E.b2;
   const T gssr = -gdw[5] * E.b2 + gdw[6] * E.b1;
-  gE.sr += gssr * E.sg * am;
-  T gam = gssr * E.sg * E.sr;
+  gE.sr += times_sign<T>(gssr, E.sg) * am;
+  T gam = times_sign<T>(gssr, E.sg) * E.sr;
   gE.As += gms * fp;
   gE.Af += -gms * sp;
   T gfp = gms * E.As, gsp = -gms * E.Af;
@@ -148,13 +211,22 @@ __device__ __forceinline__ void eig_right_vjp(const Eig<T>& E, const T* q, const
   gE.Qs += gM * fm;
   gE.Qf += -gM * sm;
   T gfm = gM * E.Qs, gsm = -gM * E.Qf;
-  const T gcfa = -gdw[1] * fm, gcsa = -gdw[1] * sm;
-  gfm += -gdw[1] * cfa;
-  gsm += -gdw[1] * csa;
-  gE.cf += gcfa * E.af;
-  gE.af += gcfa * E.cf;
-  gE.cs += gcsa * E.as;
-  gE.as += gcsa * E.cs;
+  if constexpr (sizeof(T) != 4) {
+    // c_f alpha_f = sgn(B_n) Q_f, c_s alpha_s = sgn(B_n) Q_s
+    const T gu = times_sign<T>(gdw[1], E.sg);
+    gE.Qf -= gu * fm;
+    gE.Qs -= gu * sm;
+    gfm -= gu * E.Qf;
+    gsm -= gu * E.Qs;
+  } else {
+    const T gcfa = -gdw[1] * fm, gcsa = -gdw[1] * sm;
+    gfm += -gdw[1] * cfa;
+    gsm += -gdw[1] * csa;
+    gE.cf += gcfa * E.af;
+    gE.af += gcfa * E.cf;
+    gE.cs += gcsa * E.as;
+    gE.as += gcsa * E.cs;
+  }
   gq[0] += gfp + gfm;
   gq[6] += gfp - gfm;
   gq[2] += gsp + gsm;
@@ -185,7 +257,7 @@ __device__ __forceinline__ void eig_fields_vjp(T gamma, const T* w0, T bn, const
   const T bt2 = bt2r * ir;
   const T b2 = ca2 + bt2;
   const T D = a2 - b2;
-  const T sd = tsqrt<T>(D * D + T(4) * a2 * bt2);
+  const T sd = tsqrt<T>(D * D + quad<T>(a2) * bt2);
   const T icf2 = E.rcf * E.rcf;
   const T cs2 = a2 * ca2 * icf2;
   const T sg = E.sg;
@@ -194,10 +266,10 @@ __device__ __forceinline__ void eig_fields_vjp(T gamma, const T* w0, T bn, const
   const T af = E.af, as = E.as;
   T M = T(0), N = T(0), iM = T(0), r2s = T(0);
   if (br != 0) {
-    N = T(2) * a2 * bt2;
+    N = twice<T>(a2) * bt2;
     M = br == 1 ? sd * (sd + D) : sd * (sd - D);
     iM = trcp<T>(M);
-    r2s = trcp<T>(T(2) * sd);
+    r2s = trcp<T>(twice<T>(sd));
   }
   const T ibt = gt0<T>(bt2r) ? trsqrt<T>(bt2r) : T(0);
   const bool bfree = gt0<T>(bt2r) && !(bt2r < T(1e-12) * (bn * bn + gamma * p));
@@ -207,49 +279,49 @@ __device__ __forceinline__ void eig_fields_vjp(T gamma, const T* w0, T bn, const
   T g_af = gE.af, g_as = gE.as, g_cf = gE.cf, g_cs = gE.cs;
   T g_by = T(0), g_bz = T(0), g_bn = T(0), g_p = T(0);
   // Qf = cf af sg, Qs = cs as sg, Af = a af sr, As = a as sr
-  g_cf += gE.Qf * af * sg;
-  g_af += gE.Qf * cf * sg;
-  g_cs += gE.Qs * as * sg;
-  g_as += gE.Qs * cs * sg;
+  g_cf += times_sign<T>(gE.Qf * af, sg);
+  g_af += times_sign<T>(gE.Qf * cf, sg);
+  g_cs += times_sign<T>(gE.Qs * as, sg);
+  g_as += times_sign<T>(gE.Qs * cs, sg);
   g_a += gE.Af * af * sr + gE.As * as * sr;
   g_af += gE.Af * a * sr;
   g_as += gE.As * a * sr;
   g_sr += gE.Af * a * af + gE.As * a * as;
   // a = sqrt(a2), isr = 1/sr, sr = sqrt(rho)
-  if (a > T(0)) g_a2 += g_a * T(0.5) * (a * ia2);  // 1/a = a / a^2
+  if (a > T(0)) g_a2 += half<T>(g_a) * (a * ia2);  // 1/a = a / a^2
   g_sr += -g_isr * isr * isr;
-  if (sr > T(0)) g_rho += g_sr * T(0.5) * isr;
+  if (sr > T(0)) g_rho += half<T>(g_sr) * isr;
   // b1 = by / bt, b2 = bz / bt, bt = sqrt(bt2r)
   T g_bt2r = T(0);
   if (bfree) {
     g_by += gE.b1 * ibt;
     g_bz += gE.b2 * ibt;
     const T g_bt = -(gE.b1 * by + gE.b2 * bz) * ibt * ibt;
-    g_bt2r += g_bt * T(0.5) * ibt;
+    g_bt2r += half<T>(g_bt) * ibt;
   }
   // af, as
   T g_sd = T(0), g_D = T(0), g_bt2 = T(0);
   if (br != 0) {
     // big = (sd +- D) / (2 sd), small = N / M
-    const T g_big = br == 1 ? (af > T(0) ? g_af * T(0.5) * trcp<T>(af) : T(0))
-                            : (as > T(0) ? g_as * T(0.5) * trcp<T>(as) : T(0));
-    const T g_small = br == 1 ? (as > T(0) ? g_as * T(0.5) * trcp<T>(as) : T(0))
-                              : (af > T(0) ? g_af * T(0.5) * trcp<T>(af) : T(0));
+    const T g_big = br == 1 ? (af > T(0) ? half<T>(g_af) * trcp<T>(af) : T(0))
+                            : (as > T(0) ? half<T>(g_as) * trcp<T>(as) : T(0));
+    const T g_small = br == 1 ? (as > T(0) ? half<T>(g_as) * trcp<T>(as) : T(0))
+                              : (af > T(0) ? half<T>(g_af) * trcp<T>(af) : T(0));
     const T sD = br == 1 ? T(1) : T(-1);  // big = (sd + sD D) / (2 sd)
     // d big / d sd = -sD D / (2 sd^2), d big / d D = sD / (2 sd)
     g_sd += -g_big * sD * D * r2s * r2s * T(2);
     g_D += g_big * sD * r2s;
     const T g_N = g_small * iM;
     const T g_M = -g_small * N * iM * iM;
-    g_a2 += g_N * T(2) * bt2;
-    g_bt2 += g_N * T(2) * a2;
+    g_a2 += twice<T>(g_N) * bt2;
+    g_bt2 += twice<T>(g_N) * a2;
     // M = sd (sd + sD D)
     g_sd += g_M * (T(2) * sd + sD * D);
     g_D += g_M * sD * sd;
   }
   // cs = sqrt(cs2), cf = sqrt(cf2), cs2 = a2 ca2 / cf2, cf2 = (a2 + b2 + sd)/2
-  T g_cs2 = cs > T(0) ? g_cs * T(0.5) * trcp<T>(cs) : T(0);
-  T g_cf2 = cf > T(0) ? g_cf * T(0.5) * E.rcf : T(0);
+  T g_cs2 = cs > T(0) ? half<T>(g_cs) * trcp<T>(cs) : T(0);
+  T g_cf2 = cf > T(0) ? half<T>(g_cf) * E.rcf : T(0);
   g_a2 += g_cs2 * ca2 * icf2;
   T g_ca2 = g_cs2 * a2 * icf2;
   g_cf2 += -g_cs2 * cs2 * icf2;
@@ -259,9 +331,9 @@ __device__ __forceinline__ void eig_fields_vjp(T gamma, const T* w0, T bn, const
   // sd = sqrt(D^2 + 4 a2 bt2)
   if (sd > T(0)) {
     const T g_X = g_sd * r2s;  // (sd > 0: r2s = 1/(2 sd))
-    g_D += g_X * T(2) * D;
-    g_a2 += g_X * T(4) * bt2;
-    g_bt2 += g_X * T(4) * a2;
+    g_D += twice<T>(g_X) * D;
+    g_a2 += quad<T>(g_X) * bt2;
+    g_bt2 += quad<T>(g_X) * a2;
   }
   // D = a2 - b2, b2 = ca2 + bt2, bt2 = bt2r ir, bt2r = by^2 + bz^2, ca2 = bn^2 ir
   g_a2 += g_D;
@@ -270,9 +342,9 @@ __device__ __forceinline__ void eig_fields_vjp(T gamma, const T* w0, T bn, const
   g_bt2 += g_b2;
   g_bt2r += g_bt2 * ir;
   g_ir += g_bt2 * bt2r;
-  g_by += g_bt2r * T(2) * by;
-  g_bz += g_bt2r * T(2) * bz;
-  g_bn += g_ca2 * T(2) * bn * ir;
+  g_by += twice<T>(g_bt2r) * by;
+  g_bz += twice<T>(g_bt2r) * bz;
+  g_bn += twice<T>(g_ca2) * bn * ir;
   g_ir += g_ca2 * bn * bn;
   // ia2 = 1/a2, a2 = gamma p ir, ir = 1/rho
   g_a2 += -g_ia2 * ia2 * ia2;
@@ -296,8 +368,9 @@ template <class T> struct OutlineRev { static constexpr bool v = false; };
 template <> struct OutlineRev<df> { static constexpr bool v = true; };
 template <class T> __device__ __noinline__ void ppm_one_call(const T* q, T& qm, T& qp) { ppm_one<T>(q, qm, qp); }
 template <class T>
-__device__ __noinline__ void eig_left_vjp_call(const Eig<T>& E, T ir, const T* dw, const T* gq, T* gdw, EigG<T>& gE) {
-  eig_left_vjp<T>(E, ir, dw, gq, gdw, gE);
+__device__ __noinline__ void eig_left_vjp_call(const Eig<T>& E, const T* dw, const T* gq, T* gdw, EigG<T>& gE,
+                                               EigCoefG<T>& gC) {
+  eig_left_vjp_wide<T>(E, dw, gq, gdw, gE, gC);
 }
 template <class T> __device__ __noinline__ void eig_left_call(const Eig<T>& E, const T* dw, T* q) { eig_left<T>(E, dw, q); }
 template <class T>
@@ -309,9 +382,12 @@ template <class T> __device__ __forceinline__ void eig_left_o(const Eig<T>& E, c
   if constexpr (OutlineRev<T>::v) eig_left_call<T>(E, dw, q);
   else eig_left<T>(E, dw, q);
 }
+// (gdw zero on entry)
 template <class T>
-__device__ __forceinline__ void eig_left_vjp_o(const Eig<T>& E, T ir, const T* dw, const T* gq, T* gdw, EigG<T>& gE) {
-  if constexpr (OutlineRev<T>::v) eig_left_vjp_call<T>(E, ir, dw, gq, gdw, gE);
+__device__ __forceinline__ void eig_left_vjp_o(const Eig<T>& E, T ir, const T* dw, const T* gq, T* gdw, EigG<T>& gE,
+                                               EigCoefG<T>& gC) {
+  if constexpr (OutlineRev<T>::v) eig_left_vjp_call<T>(E, dw, gq, gdw, gE, gC);
+  else if constexpr (sizeof(T) != 4) eig_left_vjp_wide<T>(E, dw, gq, gdw, gE, gC);
   else eig_left_vjp<T>(E, ir, dw, gq, gdw, gE);
 }
 template <class T>
@@ -402,9 +478,12 @@ __device__ void plmc_vjp(T gamma, T rho_floor, T p_floor, const T* wm, const T* 
     gaL[q] += T(0.5) * gaC[q];
     gaR[q] += T(0.5) * gaC[q];
   }
-  eig_left_vjp_o<T>(E, ir, dL, gaL, gdL, gE);
-  eig_left_vjp_o<T>(E, ir, dR, gaR, gdR, gE);
-  eig_left_vjp_o<T>(E, ir, dG, gaG, gdG, gE);
+  EigCoefG<T> gC;
+  gC.zero();
+  eig_left_vjp_o<T>(E, ir, dL, gaL, gdL, gE, gC);
+  eig_left_vjp_o<T>(E, ir, dR, gaR, gdR, gE, gC);
+  eig_left_vjp_o<T>(E, ir, dG, gaG, gdG, gE, gC);
+  eig_coef_vjp<T>(E, gC, gE);
 #pragma unroll
   for (int q = 0; q < 7; ++q) {
     const T pr = dL[q] * dR[q];
@@ -449,7 +528,105 @@ template <class T> __device__ __forceinline__ int d2sel4(T x, T y, T z, T t) {
   return (mcd < mab) ? scd : sab;
 }
 
+// Double and float pairs: the reverse of ppm_one_wide, with its decisions;
+// writes the cotangents of cells i-2, i-1, i+1, i+2 (gq[0], gq[1], gq[3],
+// gq[4]; the centre's deviation is identically 0).
+// lim_face: which value it returned (0: half of x, 1: v, 2: limited by y, 3: by z)
+template <class T> __device__ __forceinline__ int lim_face_sel(T x, T v, T y, T z, T& val) {
+  const T u = x - twice_f<T>(v);
+  const T ay = absv<T>(y), az = absv<T>(z);
+  const bool zy = nonneg_lt<T>(az, ay);
+  const T c = from_d<T>(1.25 / 6.0) * (zy ? az : ay);
+  if (!(pos_prod<T>(u, y) && pos_prod<T>(u, z))) {
+    val = half<T>(x);
+    return 0;
+  }
+  if (!nonneg_lt<T>(c, absv<T>(half<T>(u)))) {
+    val = v;
+    return 1;
+  }
+  val = half<T>(x) - with_sign<T>(u, c);
+  return zy ? 3 : 2;
+}
+template <class T> __device__ __forceinline__ void ppm_one_vjp_wide(const T* q, T gqm, T gqp, T* gq) {
+  const T c7 = from_d<T>(7.0 / 12.0), c1 = from_d<T>(1.0 / 12.0), c6 = from_d<T>(1.25 / 6.0);
+  const T a = q[0], b = q[1], d = q[3], e = q[4];
+  T qm = c7 * b - c1 * (a + d);
+  T qp = c7 * d - c1 * (b + e);
+  const T d2m1 = a - twice_f<T>(b);
+  const T d20 = b + d;
+  const T d2p1 = e - twice_f<T>(d);
+  int sm = 1, sp = 1;  // as lim_face_sel; 1: the value as interpolated
+  if (beyond<T>(qm, b)) {
+    T v;
+    sm = lim_face_sel<T>(b, qm, d2m1, d20, v);
+    qm = v;
+  }
+  if (beyond<T>(qp, d)) {
+    T v;
+    sp = lim_face_sel<T>(d, qp, d20, d2p1, v);
+    qp = v;
+  }
+  // reverse of the cell limiter
+  T gm = gqm, gp = gqp, g2m1 = T(0), g20 = T(0), g2p1 = T(0);
+  if (!neg_prod<T>(qm, qp) || !neg_prod<T>(b, d)) {
+    const T s = qm + qp;
+    const bool same = pos_prod<T>(s, d2m1) && pos_prod<T>(s, d20) && pos_prod<T>(s, d2p1);
+    const T am = absv<T>(d2m1), a0 = absv<T>(d20), ap = absv<T>(d2p1);
+    const bool p0 = nonneg_lt<T>(ap, a0);
+    const T m0 = p0 ? ap : a0;
+    const bool l = nonneg_lt<T>(m0, am);
+    const T t = c6 * (l ? m0 : am), sa = absv<T>(s);
+    if (!same) {
+      gm = T(0);
+      gp = T(0);
+    } else if (nonneg_lt<T>(t, sa)) {
+      // r = (C/6) d2 / s, d2 the smallest of the three
+      const T r = ratio_le1<T>(t, sa);
+      const T gr = ratio_any<T>(gqm * qm + gqp * qp, s);
+      const T gs = gr * r;
+      gm = gqm * r - gs;
+      gp = gqp * r - gs;
+      const T gd = gr * c6;
+      if (!l) g2m1 = gd;
+      else if (p0) g2p1 = gd;
+      else g20 = gd;
+    }
+  } else {
+    const bool clipm = abs_ge_twice<T>(qm, qp), clipp = abs_ge_twice<T>(qp, qm);
+    gm = clipm ? T(0) : gqm;
+    gp = clipp ? T(0) : gqp;
+    if (clipm) gp = gp - twice_f<T>(gqm);
+    if (clipp) gm = gm - twice_f<T>(gqp);
+  }
+  // reverse of the interface limiters (gm, gp become the cotangents of the
+  // interpolated values)
+  T gb = T(0), gd = T(0);
+  if (sm != 1) {
+    gb = half<T>(gm);
+    const T h = c6 * gm;
+    if (sm == 2) g2m1 -= h;
+    if (sm == 3) g20 -= h;
+    gm = T(0);
+  }
+  if (sp != 1) {
+    gd = half<T>(gp);
+    const T h = c6 * gp;
+    if (sp == 2) g20 -= h;
+    if (sp == 3) g2p1 -= h;
+    gp = T(0);
+  }
+  gq[0] = g2m1 - c1 * gm;
+  gq[1] = c7 * gm - c1 * gp + (gb + g20 - twice_f<T>(g2m1));
+  gq[3] = c7 * gp - c1 * gm + (gd + g20 - twice_f<T>(g2p1));
+  gq[4] = g2p1 - c1 * gp;
+}
+
 template <class T> __device__ void ppm_one_vjp(const T* q, T gqm, T gqp, T* gq) {
+  if constexpr (sizeof(T) != 4) {
+    ppm_one_vjp_wide<T>(q, gqm, gqp, gq);
+    return;
+  }
   const T c7 = from_d<T>(7.0 / 12.0), c1 = from_d<T>(1.0 / 12.0), c6 = from_d<T>(1.0 / 6.0);
   // forward, recording the branches
   T qm = c7 * (q[1] + q[2]) - c1 * (q[0] + q[3]);
@@ -651,6 +828,8 @@ __device__ void ppmc_vjp(T gamma, T rho_floor, T p_floor, Load wload, T bn, cons
     gqs[3][c] = gcol[4];
     // gcol[2] is the cotangent of q_0, which is identically 0 (deviation form)
   }
+  EigCoefG<T> gC;
+  gC.zero();
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     T wm[7], d[7];
@@ -658,11 +837,12 @@ __device__ void ppmc_vjp(T gamma, T rho_floor, T p_floor, Load wload, T bn, cons
 #pragma unroll
     for (int c = 0; c < 7; ++c) d[c] = wm[c] - w2[c];
     T gd[7] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-    eig_left_vjp_o<T>(E, ir, d, gqs[k], gd, gE);
+    eig_left_vjp_o<T>(E, ir, d, gqs[k], gd, gE, gC);
     put(k < 2 ? k : k + 1, gd);
 #pragma unroll
     for (int c = 0; c < 7; ++c) gw2[c] -= gd[c];
   }
+  eig_coef_vjp<T>(E, gC, gE);
   eig_fields_vjp<T>(gamma, w2, bn, E, gE, gw2, gbn);
 }
 
@@ -762,6 +942,8 @@ __device__ void ppmc_vjp_pass3(T gamma, Load wload, T bn, GqLoad gqload, EigG<T>
   Eig<T> E;
   eig_build<T>(gamma, w2, bn, E);
   const T ir = E.ir;
+  EigCoefG<T> gC;
+  gC.zero();
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     T wm[7], d[7], gq[7];
@@ -770,11 +952,12 @@ __device__ void ppmc_vjp_pass3(T gamma, Load wload, T bn, GqLoad gqload, EigG<T>
     for (int c = 0; c < 7; ++c) d[c] = wm[c] - w2[c];
     gqload(k, gq);
     T gd[7] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-    eig_left_vjp_o<T>(E, ir, d, gq, gd, gE);
+    eig_left_vjp_o<T>(E, ir, d, gq, gd, gE, gC);
     put(k < 2 ? k : k + 1, gd);
 #pragma unroll
     for (int c = 0; c < 7; ++c) gw2[c] -= gd[c];
   }
+  eig_coef_vjp<T>(E, gC, gE);
   eig_fields_vjp<T>(gamma, w2, bn, E, gE, gw2, gbn);
 }
 

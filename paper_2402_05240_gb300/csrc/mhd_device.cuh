@@ -135,8 +135,14 @@ template <> __device__ __forceinline__ double twice<double>(double v) {
   const long long x = dbits(v);
   return (x & kAbsBits) ? __longlong_as_double(x + (1LL << 52)) : v;
 }
+// (twice_f, half_f: scalings inside a sum -- a multiplication that the
+// compiler fuses with the addition, except for float pairs)
+template <class T> __device__ __forceinline__ T twice_f(T x) { return T(2) * x; }
+template <> __device__ __forceinline__ df twice_f<df>(df x) { return twice<df>(x); }
 template <class T> __device__ __forceinline__ T half(T x) { return T(0.5) * x; }
 template <> __device__ __forceinline__ df half<df>(df x) { return df(0.5f * x.hi, 0.5f * x.lo); }
+template <class T> __device__ __forceinline__ T half_f(T x) { return T(0.5) * x; }
+template <> __device__ __forceinline__ df half_f<df>(df x) { return half<df>(x); }
 template <> __device__ __forceinline__ double half<double>(double x) {
   const long long b = dbits(x), m = b & kAbsBits;
   const long long small = (m >> 1) | (b & kNegZero);  // operand or result not normal
@@ -720,8 +726,8 @@ __device__ __forceinline__ void plmc(T gamma, const T* wm, const T* w0, const T*
   eig_right<T>(E, am, dW);
 #pragma unroll
   for (int q = 0; q < 7; ++q) {
-    wl[q] = w0[q] + T(0.5) * dW[q];
-    wr[q] = w0[q] - T(0.5) * dW[q];
+    wl[q] = w0[q] + half_f<T>(dW[q]);
+    wr[q] = w0[q] - half_f<T>(dW[q]);
   }
 }
 
@@ -787,22 +793,22 @@ template <> __device__ __forceinline__ bool beyond<double>(double v, double x) {
 // The limiter for double and float pairs: the interface limiter's
 // sgn(u) min(3|u|, C|y|, C|z|)/6 as sgn(u) min(|u|/2, (C/6) min(|y|, |z|)),
 // the cell limiter's ratio min(6|s|, C m)/(6|s|) as 1 where |s| <= (C/6) m,
-// else (C/6) m / |s|, and the range tests as comparisons.
+// else (C/6) m / |s|, and the range tests as comparisons.  (An interface
+// limit (C/6) min(|y|, |z|) not below |u|/2 leaves x/2 - u/2 = v: the value stays.)
 template <class T> __device__ __forceinline__ T lim_face(T x, T v, T y, T z) {
-  const T u = x - T(2) * v;
-  T r = half<T>(x);
-  if (pos_prod<T>(u, y) && pos_prod<T>(u, z))
-    r = r - with_sign<T>(u, min_abs<T>(half<T>(u), from_d<T>(1.25 / 6.0) * min_abs<T>(y, z)));
-  return r;
+  const T u = x - twice_f<T>(v);
+  const T c = from_d<T>(1.25 / 6.0) * min_abs<T>(y, z);
+  if (!(pos_prod<T>(u, y) && pos_prod<T>(u, z))) return half<T>(x);
+  return nonneg_lt<T>(c, absv<T>(half<T>(u))) ? T(half<T>(x) - with_sign<T>(u, c)) : v;
 }
 template <class T> __device__ __forceinline__ void ppm_one_wide(const T* q, T& qm, T& qp) {
   const T c7 = from_d<T>(7.0 / 12.0), c1 = from_d<T>(1.0 / 12.0);
   const T a = q[0], b = q[1], d = q[3], e = q[4];  // cells i-2, i-1, i+1, i+2
   qm = c7 * b - c1 * (a + d);
   qp = c7 * d - c1 * (b + e);
-  const T d2m1 = a - T(2) * b;
+  const T d2m1 = a - twice_f<T>(b);
   const T d20 = b + d;
-  const T d2p1 = e - T(2) * d;
+  const T d2p1 = e - twice_f<T>(d);
   // both interfaces share one body (see ppm_one)
   const bool lm = beyond<T>(qm, b), lp = beyond<T>(qp, d);
   if (lm || lp) {
@@ -829,6 +835,12 @@ template <class T> __device__ __forceinline__ void ppm_one_wide(const T* q, T& q
     if (abs_ge_twice<T>(qm, qp)) qm = neg<T>(twice<T>(qp));
     if (abs_ge_twice<T>(qp, m0)) qp = neg<T>(twice<T>(m0));
   }
+}
+
+// a / b, b != 0
+template <class T> __device__ __forceinline__ T ratio_any(T a, T b) { return a / b; }
+template <> __device__ __forceinline__ double ratio_any<double>(double a, double b) {
+  return ratio_le1<double>(a, b);
 }
 
 // q[0..4] = characteristic deviations of cells i-2..i+2 from cell i (q[2] = 0);
