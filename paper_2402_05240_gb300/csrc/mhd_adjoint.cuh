@@ -366,7 +366,6 @@ __device__ __forceinline__ void eig_fields_vjp(T gamma, const T* w0, T bn, const
 // projections and their reverses are calls: one copy each.
 template <class T> struct OutlineRev { static constexpr bool v = false; };
 template <> struct OutlineRev<df> { static constexpr bool v = true; };
-template <class T> __device__ __noinline__ void ppm_one_call(const T* q, T& qm, T& qp) { ppm_one<T>(q, qm, qp); }
 template <class T>
 __device__ __noinline__ void eig_left_vjp_call(const Eig<T>& E, const T* dw, const T* gq, T* gdw, EigG<T>& gE,
                                                EigCoefG<T>& gC) {
@@ -378,6 +377,15 @@ __device__ __noinline__ void eig_right_vjp_call(const Eig<T>& E, const T* q, con
   eig_right_vjp<T>(E, q, gdw, gq, gE);
 }
 // the calls above where OutlineRev<T> holds, else the inlined functions
+template <class T> __device__ __forceinline__ void ppm_one_o(const T* col, T& qm, T& qp) {
+  if constexpr (sizeof(T) != 4) {
+    const LimitedPair<T> r = ppm_one_call<T>(col[0], col[1], col[3], col[4]);
+    qm = r.m;
+    qp = r.p;
+  } else {
+    ppm_one<T>(col, qm, qp);
+  }
+}
 template <class T> __device__ __forceinline__ void eig_left_o(const Eig<T>& E, const T* dw, T* q) {
   if constexpr (OutlineRev<T>::v) eig_left_call<T>(E, dw, q);
   else eig_left<T>(E, dw, q);
@@ -533,7 +541,7 @@ template <class T> __device__ __forceinline__ int d2sel4(T x, T y, T z, T t) {
 // gq[4]; the centre's deviation is identically 0).
 // lim_face: which value it returned (0: half of x, 1: v, 2: limited by y, 3: by z)
 template <class T> __device__ __forceinline__ int lim_face_sel(T x, T v, T y, T z, T& val) {
-  const T u = x - twice_f<T>(v);
+  const T u = sub_twice<T>(x, v);
   const T ay = absv<T>(y), az = absv<T>(z);
   const bool zy = nonneg_lt<T>(az, ay);
   const T c = from_d<T>(1.25 / 6.0) * (zy ? az : ay);
@@ -553,9 +561,9 @@ template <class T> __device__ __forceinline__ void ppm_one_vjp_wide(const T* q, 
   const T a = q[0], b = q[1], d = q[3], e = q[4];
   T qm = c7 * b - c1 * (a + d);
   T qp = c7 * d - c1 * (b + e);
-  const T d2m1 = a - twice_f<T>(b);
+  const T d2m1 = sub_twice<T>(a, b);
   const T d20 = b + d;
-  const T d2p1 = e - twice_f<T>(d);
+  const T d2p1 = sub_twice<T>(e, d);
   int sm = 1, sp = 1;  // as lim_face_sel; 1: the value as interpolated
   if (beyond<T>(qm, b)) {
     T v;
@@ -596,8 +604,8 @@ template <class T> __device__ __forceinline__ void ppm_one_vjp_wide(const T* q, 
     const bool clipm = abs_ge_twice<T>(qm, qp), clipp = abs_ge_twice<T>(qp, qm);
     gm = clipm ? T(0) : gqm;
     gp = clipp ? T(0) : gqp;
-    if (clipm) gp = gp - twice_f<T>(gqm);
-    if (clipp) gm = gm - twice_f<T>(gqp);
+    if (clipm) gp = sub_twice<T>(gp, gqm);
+    if (clipp) gm = sub_twice<T>(gm, gqp);
   }
   // reverse of the interface limiters (gm, gp become the cotangents of the
   // interpolated values)
@@ -617,8 +625,8 @@ template <class T> __device__ __forceinline__ void ppm_one_vjp_wide(const T* q, 
     gp = T(0);
   }
   gq[0] = g2m1 - c1 * gm;
-  gq[1] = c7 * gm - c1 * gp + (gb + g20 - twice_f<T>(g2m1));
-  gq[3] = c7 * gp - c1 * gm + (gd + g20 - twice_f<T>(g2p1));
+  gq[1] = c7 * gm - c1 * gp + sub_twice<T>(gb + g20, g2m1);
+  gq[3] = c7 * gp - c1 * gm + sub_twice<T>(gd + g20, g2p1);
   gq[4] = g2p1 - c1 * gp;
 }
 
@@ -754,8 +762,27 @@ template <class T> __device__ void ppm_one_vjp(const T* q, T gqm, T gqp, T* gq) 
   gq[2] += gq2;
 }
 
-template <class T> __device__ __noinline__ void ppm_one_vjp_call(const T* q, T gqm, T gqp, T* gq) {
-  ppm_one_vjp<T>(q, gqm, gqp, gq);
+// (double and float pairs: a call with its operands in registers)
+template <class T> struct StencilCotangent {
+  T a, b, d, e;
+};
+template <class T>
+__device__ __noinline__ StencilCotangent<T> ppm_one_vjp_call(T a, T b, T d, T e, T gqm, T gqp) {
+  const T q[5] = {a, b, T(0), d, e};
+  T g[5];
+  ppm_one_vjp<T>(q, gqm, gqp, g);
+  return StencilCotangent<T>{g[0], g[1], g[3], g[4]};
+}
+template <class T> __device__ __forceinline__ void ppm_one_vjp_o(const T* q, T gqm, T gqp, T* gq) {
+  if constexpr (sizeof(T) != 4) {
+    const StencilCotangent<T> r = ppm_one_vjp_call<T>(q[0], q[1], q[3], q[4], gqm, gqp);
+    gq[0] = r.a;
+    gq[1] = r.b;
+    gq[3] = r.d;
+    gq[4] = r.e;
+  } else {
+    ppm_one_vjp<T>(q, gqm, gqp, gq);
+  }
 }
 
 // Reverse of PPMC for one cell.  wload(m, w7) loads the directional state of
@@ -787,8 +814,7 @@ __device__ void ppmc_vjp(T gamma, T rho_floor, T p_floor, Load wload, T bn, cons
   for (int c = 0; c < 7; ++c) {
     const T col[5] = {qs[0][c], qs[1][c], T(0), qs[2][c], qs[3][c]};
     T qm, qp;
-    if constexpr (OutlineRev<T>::v) ppm_one_call<T>(col, qm, qp);
-    else ppm_one<T>(col, qm, qp);
+    ppm_one_o<T>(col, qm, qp);
     dm[c] = qm;
     dp[c] = qp;
   }
@@ -820,8 +846,7 @@ __device__ void ppmc_vjp(T gamma, T rho_floor, T p_floor, Load wload, T bn, cons
   for (int c = 0; c < 7; ++c) {
     const T col[5] = {qs[0][c], qs[1][c], T(0), qs[2][c], qs[3][c]};
     T gcol[5] = {T(0), T(0), T(0), T(0), T(0)};
-    if constexpr (OutlineRev<T>::v) ppm_one_vjp_call<T>(col, gdm[c], gdp[c], gcol);
-    else ppm_one_vjp<T>(col, gdm[c], gdp[c], gcol);
+    ppm_one_vjp_o<T>(col, gdm[c], gdp[c], gcol);
     gqs[0][c] = gcol[0];
     gqs[1][c] = gcol[1];
     gqs[2][c] = gcol[3];
@@ -886,8 +911,7 @@ __device__ void ppmc_vjp_pass1(T gamma, T rho_floor, T p_floor, Load wload, T bn
     for (int c = 0; c < 7; ++c) {
       const T col[5] = {qs[0][c], qs[1][c], T(0), qs[2][c], qs[3][c]};
       T qm, qp;
-      if constexpr (OutlineRev<T>::v) ppm_one_call<T>(col, qm, qp);
-      else ppm_one<T>(col, qm, qp);
+      ppm_one_o<T>(col, qm, qp);
       dm[c] = qm;
       dp[c] = qp;
     }
@@ -925,8 +949,7 @@ __device__ void ppmc_vjp_pass2(T gamma, Load wload, T bn, const T* gdm, const T*
   for (int c = 0; c < 7; ++c) {
     const T col[5] = {qs[0][c], qs[1][c], T(0), qs[2][c], qs[3][c]};
     T gcol[5] = {T(0), T(0), T(0), T(0), T(0)};
-    if constexpr (OutlineRev<T>::v) ppm_one_vjp_call<T>(col, gdm[c], gdp[c], gcol);
-    else ppm_one_vjp<T>(col, gdm[c], gdp[c], gcol);
+    ppm_one_vjp_o<T>(col, gdm[c], gdp[c], gcol);
     gq[0][c] = gcol[0];
     gq[1][c] = gcol[1];
     gq[2][c] = gcol[3];

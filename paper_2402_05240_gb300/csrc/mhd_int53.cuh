@@ -1,5 +1,5 @@
-// mhd_int53.cuh -- reciprocal, square root and reciprocal square root of
-// doubles on the integer and FP32 pipes.
+// mhd_int53.cuh -- reciprocal, square root, reciprocal square root and product
+// of doubles on the integer and FP32 pipes.
 //
 // GB300 issues one FP64 warp instruction per SM every 16 clocks against four
 // of any other kind per clock, so an FP64 instruction costs 64 issue slots
@@ -96,6 +96,22 @@ MHD_INT_HD uint64_t sqrt_sig(uint64_t M, int odd, float seed) {
   return q + (rem > (int64_t)q) - (rem <= -(int64_t)q);
 }
 
+// Product of two 53-bit significands a, b in [2^52, 2^53): the 53-bit
+// significand q in [2^52, 2^53] of the product rounded to nearest even; big:
+// the product of the two values in [1, 2) is 2 or more.
+MHD_INT_HD uint64_t mul_sig(uint64_t a, uint64_t b, int& big) {
+  const uint64_t A = a << 10, B = b << 11;  // A B in [2^125, 2^127)
+  const uint32_t al = (uint32_t)A, ah = (uint32_t)(A >> 32), bl = (uint32_t)B, bh = (uint32_t)(B >> 32);
+  const uint64_t p0 = (uint64_t)al * bl;
+  const uint64_t p1 = (uint64_t)al * bh + (uint32_t)(p0 >> 32);
+  const uint64_t p2 = (uint64_t)ah * bl + (uint32_t)p1;
+  uint64_t hi = (uint64_t)ah * bh + (p1 >> 32) + (p2 >> 32);
+  hi |= ((uint32_t)p2 | (uint32_t)p0) != 0;  // sticky
+  big = (int)(hi >> 62);
+  const int sh = 9 + big;
+  return (hi + (((1ull << sh) >> 1) - 1 + ((hi >> sh) & 1))) >> sh;
+}
+
 #if defined(__CUDACC__)
 
 __device__ __forceinline__ float rcp_seed(float x) {
@@ -109,13 +125,6 @@ __device__ __forceinline__ float rsqrt_seed(float x) {
   return r;
 }
 
-// operands outside the range below (zero, subnormal, infinite, NaN, negative
-// under a root, results that are not normal): the library function, called
-// only in warps where a lane needs it
-static __device__ __noinline__ double rcp_other(double x) { return __drcp_rn(x); }
-static __device__ __noinline__ double sqrt_other(double x) { return __dsqrt_rn(x); }
-static __device__ __noinline__ double rsqrt_other(double x) { return rsqrt(x); }
-
 __device__ __forceinline__ uint64_t sig53(int hi, int lo) {
   return ((uint64_t)(uint32_t)((hi & 0xfffff) | 0x100000) << 32) | (uint32_t)lo;
 }
@@ -124,43 +133,75 @@ __device__ __forceinline__ uint32_t frac23(int hi, int lo) {
   return __funnelshift_l((uint32_t)lo, (uint32_t)hi, 3) & 0x7fffffu;
 }
 
-__device__ __forceinline__ double rcp_int(double x) {
+// The functions on doubles.  bad is set where an operand or the result is
+// outside the range they cover (subnormal, infinite, NaN, negative under a
+// root, zero under a reciprocal): the value returned there means nothing.
+__device__ __forceinline__ double rcp_try(double x, bool& bad) {
   const int hi = __double2hiint(x), lo = __double2loint(x);
   const int ex = (hi >> 20) & 0x7ff;
-  const bool ok = (unsigned)(ex - 1) < 2044u;
+  bad |= (unsigned)(ex - 1) >= 2044u;
   const uint64_t q = rcp_sig(sig53(hi, lo), rcp_seed(__uint_as_float(0x3f800000u | frac23(hi, lo))));
   const int rh = (int)(uint32_t)(q >> 32) + ((2044 - ex) << 20);
-  double r = __hiloint2double(rh | (hi & (int)0x80000000), (int)(uint32_t)q);
-  if (__any_sync(__activemask(), !ok)) {
-    if (!ok) r = rcp_other(x);
-  }
-  return r;
+  return __hiloint2double(rh | (hi & (int)0x80000000), (int)(uint32_t)q);
 }
-
-__device__ __forceinline__ double rsqrt_int(double x) {
+__device__ __forceinline__ double rsqrt_try(double x, bool& bad) {
   const int hi = __double2hiint(x), lo = __double2loint(x);
-  const bool ok = (unsigned)(hi - 0x00100000) < 0x7fe00000u;  // positive and normal
+  bad |= (unsigned)(hi - 0x00100000) >= 0x7fe00000u;  // not positive and normal
   const int ex = hi >> 20, odd = (ex & 1) ^ 1, k = (ex - 1023 - odd) >> 1;
   const float seed = rsqrt_seed(__uint_as_float((0x3f800000u + ((unsigned)odd << 23)) | frac23(hi, lo)));
   const uint64_t q = rsqrt_sig(sig53(hi, lo), odd, seed);
-  double r = __hiloint2double((int)(uint32_t)(q >> 32) + ((1021 - k) << 20), (int)(uint32_t)q);
-  if (__any_sync(__activemask(), !ok)) {
-    if (!ok) r = rsqrt_other(x);
-  }
-  return r;
+  return __hiloint2double((int)(uint32_t)(q >> 32) + ((1021 - k) << 20), (int)(uint32_t)q);
 }
-
-__device__ __forceinline__ double sqrt_int(double x) {
+__device__ __forceinline__ double sqrt_try(double x, bool& bad) {
   const int hi = __double2hiint(x), lo = __double2loint(x);
   const bool zero = ((hi & 0x7fffffff) | lo) == 0;
-  const bool ok = zero | ((unsigned)(hi - 0x00100000) < 0x7fe00000u);
+  bad |= !zero & ((unsigned)(hi - 0x00100000) >= 0x7fe00000u);
   const int ex = hi >> 20, odd = (ex & 1) ^ 1, k = (ex - 1023 - odd) >> 1;
   const float seed = rsqrt_seed(__uint_as_float((0x3f800000u + ((unsigned)odd << 23)) | frac23(hi, lo)));
   const uint64_t q = sqrt_sig(sig53(hi, lo), odd, seed);
-  double r = __hiloint2double((int)(uint32_t)(q >> 32) + ((1022 + k) << 20), (int)(uint32_t)q);
-  r = zero ? x : r;
-  if (__any_sync(__activemask(), !ok)) {
-    if (!ok) r = sqrt_other(x);
+  const double r = __hiloint2double((int)(uint32_t)(q >> 32) + ((1022 + k) << 20), (int)(uint32_t)q);
+  return zero ? x : r;
+}
+// a b (the IEEE product)
+__device__ __forceinline__ double mul_try(double a, double b, bool& bad) {
+  const int ha = __double2hiint(a), la = __double2loint(a), hb = __double2hiint(b), lb = __double2loint(b);
+  const int ea = (ha >> 20) & 0x7ff, eb = (hb >> 20) & 0x7ff;
+  int big;
+  const uint64_t q = mul_sig(sig53(ha, la), sig53(hb, lb), big);
+  const int e = ea + eb - 1023 + big;
+  const bool zero = (((ha << 1) | la) == 0) | (((hb << 1) | lb) == 0);
+  bad |= ((unsigned)(ea - 1) >= 2046u) | ((unsigned)(eb - 1) >= 2046u) | ((unsigned)(e - 1) >= 2045u) ? !(zero & (ea < 2047) & (eb < 2047)) : false;
+  const int s = (ha ^ hb) & (int)0x80000000;
+  const int rh = (int)(uint32_t)(q >> 32) + ((e - 1) << 20);
+  return __hiloint2double((zero ? 0 : rh) | s, zero ? 0 : (int)(uint32_t)q);
+}
+
+// For every operand: outside that range the library function, called only in
+// warps where a lane needs it.
+static __device__ __noinline__ double rcp_other(double x) { return __drcp_rn(x); }
+static __device__ __noinline__ double sqrt_other(double x) { return __dsqrt_rn(x); }
+static __device__ __noinline__ double rsqrt_other(double x) { return rsqrt(x); }
+__device__ __forceinline__ double rcp_int(double x) {
+  bool bad = false;
+  double r = rcp_try(x, bad);
+  if (__any_sync(__activemask(), bad)) {
+    if (bad) r = rcp_other(x);
+  }
+  return r;
+}
+__device__ __forceinline__ double rsqrt_int(double x) {
+  bool bad = false;
+  double r = rsqrt_try(x, bad);
+  if (__any_sync(__activemask(), bad)) {
+    if (bad) r = rsqrt_other(x);
+  }
+  return r;
+}
+__device__ __forceinline__ double sqrt_int(double x) {
+  bool bad = false;
+  double r = sqrt_try(x, bad);
+  if (__any_sync(__activemask(), bad)) {
+    if (bad) r = sqrt_other(x);
   }
   return r;
 }

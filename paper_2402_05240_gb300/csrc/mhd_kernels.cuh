@@ -446,20 +446,20 @@ template <class T> __device__ __forceinline__ void floor_face(const Grid& g, T* 
   w[4] = max_pos<T>(w[4], from_d<T>(g.p_floor));
 }
 
-// blocks of 128 threads per SM requested from the register allocator (4:
-// at most 128 registers per thread).  The double and double-float PPMC and
-// the double PLMC kernels fit 128 registers without spilling; the
-// double-float PLMC kernel spills 40 bytes there and still runs 9 % faster
-// than at 3 blocks (168 registers, no spill): its dependent float-pair
-// chains need the extra warps.  (The double-float flux kernels, 112-119
-// registers, lose 2 % at 5 blocks with 40-68 bytes of spill; the double PLMC
-// kernel, 108 registers, loses 5 % at 5 blocks, 96 registers.)
-template <class T, int RECON> struct ReconMinBlocks { static constexpr int v = 4; };
+// blocks of 128 threads per SM requested from the register allocator.  4 (at
+// most 128 registers per thread) for float pairs and float: the float-pair
+// kernels lose 9 % (PPMC) and 12 % (PLMC) at 3 blocks, their dependent chains
+// need the extra warps.  3 (168 registers) for the double PLMC and PPMC
+// kernels, which interleave integer-pipe products with the FP64 pipe: at 4
+// blocks they spill 0.5 KB (256^3: 22.4 and 40.6 ms against 21.4 and 38.6 ms).
+template <class T, int RECON> struct ReconMinBlocks {
+  static constexpr int v = std::is_same<T, double>::value && (RECON == 1 || RECON == 2) ? 3 : 4;
+};
 
 // interface states of cell p along A (Step 6): wl = W_{L,i+1/2} (the cell's
 // state at its upper face), wr = W_{R,i-1/2} (at its lower face), floored
-template <class T, int RECON, int A>
-__device__ __forceinline__ void recon_cell(const Grid& g, const Fields<const T, 8>& W, const Cell& p, T* wl, T* wr) {
+template <class T, int RECON, int A, class O>
+__device__ __forceinline__ void recon_cell_with(O& o, const Grid& g, const Fields<const T, 8>& W, const Cell& p, T* wl, T* wr) {
   const int c = p.c;
   const T bn = ldg(W.f[5 + A] + c);
   if (RECON == 0) {
@@ -471,16 +471,41 @@ __device__ __forceinline__ void recon_cell(const Grid& g, const Fields<const T, 
     load_dir<A>(W, c + p.m[A], wm);
     load_dir<A>(W, c, w0);
     load_dir<A>(W, c + p.p[A], wp);
-    if (RECON == 1) plmc<T>(from_d<T>(g.gamma), wm, w0, wp, bn, wl, wr);
+    if (RECON == 1) plmc<T>(o, from_d<T>(g.gamma), wm, w0, wp, bn, wl, wr);
     else plm_prim<T>(wm, w0, wp, wl, wr);
   } else {
     T w[5][7];
 #pragma unroll
     for (int s = -2; s <= 2; ++s) load_dir<A>(W, c + off<A>(g, p, s), w[s + 2]);
-    ppmc<T>(from_d<T>(g.gamma), w, bn, wl, wr);
+    ppmc<T>(o, from_d<T>(g.gamma), w, bn, wl, wr);
   }
   floor_face<T>(g, wl);
   floor_face<T>(g, wr);
+}
+
+template <class T, int RECON, int A>
+__device__ __noinline__ void recon_cell_again(const Grid& g, const Fields<const T, 8>& W, const Cell& p, T* wl, T* wr) {
+  Ops<T> o;
+  recon_cell_with<T, RECON, A>(o, g, W, p, wl, wr);
+}
+template <class T, int RECON, int A>
+__device__ __forceinline__ void recon_cell(const Grid& g, const Fields<const T, 8>& W, const Cell& p, T* wl, T* wr) {
+  TryOps<T> o;
+  recon_cell_with<T, RECON, A>(o, g, W, p, wl, wr);
+  if constexpr (std::is_same<T, double>::value && (RECON == 1 || RECON == 2)) {
+    if (__any_sync(__activemask(), o.bad)) {
+      if (o.bad) {
+        const Cell pc = p;
+        T a[7], b[7];
+        recon_cell_again<T, RECON, A>(g, W, pc, a, b);
+#pragma unroll
+        for (int q = 0; q < 7; ++q) {
+          wl[q] = a[q];
+          wr[q] = b[q];
+        }
+      }
+    }
+  }
 }
 
 template <class T, int RECON, int A>
@@ -599,11 +624,50 @@ template <> __device__ __forceinline__ double upwind<double>(double m, double fl
   const long long b = dbits(m);
   const bool z = (b & kAbsBits) == 0;
   const bool lo = b > 0;
-  double d = (lo ? flo : fhi) - (lo ? rlo : rhi);
+  double d = pick<double>(lo, flo, fhi) - pick<double>(lo, rlo, rhi);
   if (__any_sync(__activemask(), z)) {
     if (z) d = upwind_mean(flo, rlo, fhi, rhi);
   }
   return d;
+}
+// f + r in the place of f - r
+template <class T> __device__ __forceinline__ T upwind_plus(T m, T flo, T rlo, T fhi, T rhi) {
+  const T lo = flo + rlo, hi = fhi + rhi;
+  return m > T(0) ? lo : (m < T(0) ? hi : half<T>(lo + hi));
+}
+template <> __device__ __forceinline__ double upwind_plus<double>(double m, double flo, double rlo, double fhi,
+                                                                  double rhi) {
+  const long long b = dbits(m);
+  const bool z = (b & kAbsBits) == 0;
+  const bool lo = b > 0;
+  double d = pick<double>(lo, flo, fhi) + pick<double>(lo, rlo, rhi);
+  if (__any_sync(__activemask(), z)) {
+    if (z) d = upwind_mean(flo, neg<double>(rlo), fhi, neg<double>(rhi));
+  }
+  return d;
+}
+
+// The edge field from the induction fluxes b (of B_C through the B faces of
+// cells 0 and 0 + e_C; the electric field is -b) and c (of B_B through the C
+// faces of cells 0 and 0 + e_B), their mass fluxes mb, mc and the reference
+// fields of the four cells.  Double and float pairs sum the -b terms as they
+// are and subtract them once, so no value is negated (a negation that feeds a
+// selection is an FP64-pipe addition): 11 additions per edge against 16, and
+// at 256^3 1.06 ms per launch against 1.53 (FP64).
+template <class T>
+__device__ __forceinline__ T edge_of(T b0, T bc, T c0, T cb, T mb0, T mbc, T mc0, T mcb, T r00, T rb, T rc, T rbc) {
+  if constexpr (sizeof(T) != 4) {
+    const T C = (upwind<T>(mbc, c0, rc, cb, rbc) + upwind<T>(mb0, c0, r00, cb, rb)) + (cb + c0);
+    const T B = (upwind_plus<T>(mcb, b0, rb, bc, rbc) + upwind_plus<T>(mc0, b0, r00, bc, rc)) + (bc + b0);
+    return quarter<T>(C - B);
+  }
+  const T bf0 = -b0, bfc = -bc;
+  const T avg = T(0.25) * (bfc + bf0 + cb + c0);
+  const T Dcp = upwind<T>(mbc, c0, rc, cb, rbc);
+  const T Dcm = upwind<T>(mb0, c0, r00, cb, rb);
+  const T Dbp = upwind<T>(mcb, bf0, rb, bfc, rbc);
+  const T Dbm = upwind<T>(mc0, bf0, r00, bfc, rc);
+  return avg + T(0.25) * (Dcp + Dcm + Dbp + Dbm);
 }
 
 template <class T, int A, bool REF>
@@ -624,16 +688,9 @@ __device__ __forceinline__ T edge_field(const Grid& g, const Fields<const T, 8>&
       return cell_ref<T, A>(w8);
     }
   };
-  const T bf0 = neg<T>(ldg(Fbb + q00)), bfc = neg<T>(ldg(Fbb + qc));
-  const T cf0 = ldg(Fcb + q00), cfb = ldg(Fcb + qb);
-  const T r00 = ref(q00), rb = ref(qb), rc = ref(qc), rbc = ref(qbc);
-  const T avg = T(0.25) * (bfc + bf0 + cfb + cf0);
-  const T Dcp = upwind<T>(ldg(Fbm + qc), cf0, rc, cfb, rbc);
-  const T Dcm = upwind<T>(ldg(Fbm + q00), cf0, r00, cfb, rb);
-  const T Dbp = upwind<T>(ldg(Fcm + qb), bf0, rb, bfc, rbc);
-  const T Dbm = upwind<T>(ldg(Fcm + q00), bf0, r00, bfc, rc);
-  if constexpr (sizeof(T) != 4) return quarter<T>(((bfc + bf0) + (cfb + cf0)) + ((Dcp + Dcm) + (Dbp + Dbm)));
-  return avg + T(0.25) * (Dcp + Dcm + Dbp + Dbm);
+  const T b0 = ldg(Fbb + q00), bc = ldg(Fbb + qc), c0 = ldg(Fcb + q00), cb = ldg(Fcb + qb);
+  return edge_of<T>(b0, bc, c0, cb, ldg(Fbm + q00), ldg(Fbm + qc), ldg(Fcm + q00), ldg(Fcm + qb), ref(q00), ref(qb),
+                    ref(qc), ref(qbc));
 }
 
 // REF: the cells' reference fields come from Er (written with W), else from W
@@ -678,16 +735,8 @@ __device__ __forceinline__ T edge_field_r(const Grid& g, const T* __restrict__ W
       return cell_ref<T, A>(w8);
     }
   };
-  const T bf0 = neg<T>(Fb[5 * N + q00]), bfc = neg<T>(Fb[5 * N + qc]);
-  const T cf0 = Fc[6 * N + q00], cfb = Fc[6 * N + qb];
-  const T r00 = ref(q00), rb = ref(qb), rc = ref(qc), rbc = ref(qbc);
-  const T avg = T(0.25) * (bfc + bf0 + cfb + cf0);
-  const T Dcp = upwind<T>(Fb[qc], cf0, rc, cfb, rbc);
-  const T Dcm = upwind<T>(Fb[q00], cf0, r00, cfb, rb);
-  const T Dbp = upwind<T>(Fc[qb], bf0, rb, bfc, rbc);
-  const T Dbm = upwind<T>(Fc[q00], bf0, r00, bfc, rc);
-  if constexpr (sizeof(T) != 4) return quarter<T>(((bfc + bf0) + (cfb + cf0)) + ((Dcp + Dcm) + (Dbp + Dbm)));
-  return avg + T(0.25) * (Dcp + Dcm + Dbp + Dbm);
+  return edge_of<T>(Fb[5 * N + q00], Fb[5 * N + qc], Fc[6 * N + q00], Fc[6 * N + qb], Fb[q00], Fb[qc], Fc[q00], Fc[qb],
+                    ref(q00), ref(qb), ref(qc), ref(qbc));
 }
 
 template <class T, bool REF>

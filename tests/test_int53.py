@@ -64,3 +64,37 @@ def harness(tmp_path_factory):
 def test_rounding_for_every_seed_in_the_bound(harness, kind):
     out = subprocess.run([harness, str(kind)], check=True, capture_output=True, text=True).stdout.split()
     assert [int(v) for v in out] == [0, 0, 0]
+
+
+PRODUCTS = r"""
+#include <cstdio>
+#include <random>
+#include "mhd_int53.cuh"
+using namespace mhd;
+int main() {
+  std::mt19937_64 g(5);
+  const uint64_t all = (1ull << 52) - 1;
+  long bad = 0;
+  for (long it = 0; it < 4000000; ++it) {
+    uint64_t fa = g() & all, fb = g() & all;
+    if (it % 8 == 1) fa &= 0xffff;                                    // 1 + ulps
+    if (it % 8 == 2) fa = (fa >> 26) << 26, fb = (fb >> 26) << 26;      // exact products
+    if (it % 8 == 3) fa = (fa >> 30) << 30, fb = (fb >> 20) << 20;      // ties
+    if (it % 8 == 4) fa |= all ^ 0xff, fb |= all ^ 0xff;                // carries out of the significand
+    if (it % 8 == 5) fa = 0;
+    const uint64_t a = (1ull << 52) | fa, b = (1ull << 52) | fb;
+    int big;
+    const uint64_t q = mul_sig(a, b, big);
+    bad += (double)q * 0x1p-52 * (big ? 2 : 1) != ((double)a * 0x1p-52) * ((double)b * 0x1p-52);
+  }
+  printf("%ld\n", bad);
+  return 0;
+}
+"""
+
+
+def test_products_are_ieee(tmp_path):
+    src, exe = tmp_path / "p.cpp", tmp_path / "p"
+    src.write_text(PRODUCTS)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    assert subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.strip() == "0"
