@@ -10,7 +10,16 @@ void launch_set_dt(const Grid& g, double* dt_cur, double value, cudaStream_t s) 
 }
 void launch_finish_dt(const Grid& g, unsigned long long* dtbits, double* dt_cur, double* dt_log, int step,
                       unsigned* flags, double t_end, cudaStream_t s) {
-  k_finish_dt<<<1, 1, 0, s>>>(g, dtbits, dt_cur, dt_log, step, flags, t_end);
+  cudaLaunchAttribute at = {};  // early (grid_wait)
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(1);
+  c.blockDim = dim3(1);
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, k_finish_dt, g, dtbits, dt_cur, dt_log, step, flags, t_end);
 }
 static int copy_blocks(long long n) {
   const long long b = (n + 255) / 256;

@@ -259,9 +259,8 @@ template <> __device__ __forceinline__ double ratio_le1<double>(double a, double
 // anyway): on the integer pipes a product costs about 38 issue slots against
 // the 64 of an FP64 instruction, and the FP64 pipe has the less idle time.
 // Measured at 256^3, FP64: Riemann kernels (30 products of 120 operations) 10.9
-// -> 9.1 ms, PLMC reconstruction (40 of 250) 23.9 -> 21.4 ms, PPMC 41.4 -> 38.6 ms.
-// The products of the projections and of the limiter stay on the FP64 pipe:
-// more of them spill registers and outgrow the instruction cache (45.8 ms).
+// -> 9.1 ms, PLMC reconstruction 23.9 -> 20.2 ms, PPMC 41.4 -> 33.2 ms (31
+// products of the eigensystem and 8 of each projection, as calls: CallOps).
 template <class T> struct Ops {
   static constexpr bool bad = false;
   __device__ __forceinline__ T rcp(T x) { return trcp<T>(x); }
@@ -282,6 +281,28 @@ template <> struct TryOps<double> {
     return __longlong_as_double(b ? b + (2LL << 52) : b);
   }
   __device__ __forceinline__ double mul(double a, double b) { return mul_try(a, b, bad); }
+};
+
+// TryOps with the product as a call, for the reconstruction: inlined, its
+// products spill registers and outgrow the instruction cache, so only those of
+// the eigensystem paid; as a call (operands and result in registers) those of
+// the projections do too.
+struct TryValue {
+  double v;
+  int bad;
+};
+static __device__ __noinline__ TryValue mul_try_call(double a, double b) {
+  bool bad = false;
+  const double v = mul_try(a, b, bad);
+  return TryValue{v, bad};
+}
+template <class T> struct CallOps : TryOps<T> {};
+template <> struct CallOps<double> : TryOps<double> {
+  __device__ __forceinline__ double mul(double a, double b) {
+    const TryValue r = mul_try_call(a, b);
+    bad |= r.bad != 0;
+    return r.v;
+  }
 };
 
 // ------------------------------------------------- primitives (Sec. 2.2.1) --
@@ -693,12 +714,12 @@ template <class T, class O> __device__ __forceinline__ void eig_left(O& o, const
     const T h1 = half<T>(E.b1), h2 = half<T>(E.b2);
     const T z = times_sign<T>(E.isr, E.sg);
     const T z1 = o.mul(h1, z), z2 = o.mul(h2, z);
-    const T bv = times_sign<T>(E.b1 * dw[2] + E.b2 * dw[3], E.sg);
-    const T bb = E.b1 * dw[5] + E.b2 * dw[6];
-    const T Xf = fp * dw[4] + fb * bb, Yf = su * bv - fu * dw[1];
-    const T Xs = sp * dw[4] - sb * bb, Ys = su * dw[1] + fu * bv;
-    const T Z = h1 * dw[3] - h2 * dw[2];
-    const T Zb = z1 * dw[6] - z2 * dw[5];
+    const T bv = times_sign<T>(o.mul(E.b1, dw[2]) + E.b2 * dw[3], E.sg);
+    const T bb = o.mul(E.b1, dw[5]) + E.b2 * dw[6];
+    const T Xf = o.mul(fp, dw[4]) + fb * bb, Yf = o.mul(su, bv) - fu * dw[1];
+    const T Xs = o.mul(sp, dw[4]) - sb * bb, Ys = o.mul(su, dw[1]) + fu * bv;
+    const T Z = o.mul(h1, dw[3]) - h2 * dw[2];
+    const T Zb = o.mul(z1, dw[6]) - z2 * dw[5];
     q[0] = Xf + Yf;
     q[1] = Z + Zb;
     q[2] = Xs - Ys;
@@ -1014,7 +1035,7 @@ template <class T> __device__ __forceinline__ void ppm_one(const T* q, T& qm, T&
 // The limiter as a call (double and float pairs): seven inlined copies outgrow
 // the instruction cache (1.2 warps stalled on instruction fetch per issue in
 // the FP64 kernel).  Measured at 256^3: float pairs 10.0 -> 9.4 ms, FP64 45.1 ->
-// 40.6 ms with the products of the eigensystem on the integer pipes.
+// 40.6 ms with the inlined products of the eigensystem.
 template <class T> struct LimitedPair {
   T m, p;
 };

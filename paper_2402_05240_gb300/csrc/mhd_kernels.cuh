@@ -88,6 +88,34 @@ inline dim3 grid3_of(const Grid& g) {
   return dim3(d.x, d.y, 3 * d.z);
 }
 
+// Early launch of the step kernels (programmatic dependent launch).  Every
+// step kernel waits here, before its first access to memory, for the kernel
+// before it to finish with its writes visible, and only then lets the next one
+// be scheduled: at most one launch is ahead, so nothing that a kernel reads was
+// read before by a kernel still running beside it, except where that kernel
+// updates in place (k_update_full), after which k_prim is launched the
+// ordinary way.  Launched without the attribute, both instructions do nothing.
+// The cell index passes through an empty statement after the wait, so no load
+// can be moved above it.  Measured per PPMC step, ordinary / early launch:
+// FP32-bulk 16^3 48 / 32 us, 32^3 55 / 40, 64^3 141 / 124, 128^3 818 / 798, 256^3
+// 5767 / 5734; float pairs 32^3 105 / 86; FP64 32^3 232 / 218 us.
+__device__ __forceinline__ void grid_wait(int& c) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("" : "+r"(c)::"memory");
+}
+__device__ __forceinline__ Cell step_cell(const Grid& g, int k) {
+  Cell p = thread_cell(g, k);
+  grid_wait(p.c);
+  return p;
+}
+__device__ __forceinline__ Cell step_cell(const Grid& g) { return step_cell(g, blockIdx.z); }
+__device__ __forceinline__ CellIdx step_cell_idx(const Grid& g) {
+  CellIdx c = cell_of_thread(g);
+  grid_wait(c.i);
+  return c;
+}
+
 // offset from cell p to p + s e_A (periodic), |s| < n[A]
 template <int A> __device__ __forceinline__ int off(const Grid& g, const Cell& p, int s) {
   if (s == 0) return 0;
@@ -220,18 +248,11 @@ template <class T> __device__ __forceinline__ void store_w(const Fields<T, 8>& W
   for (int f = 0; f < 8; ++f) W.f[f][c] = w8[f];
 }
 
-// x / 4 for x >= 0, exact: on the exponent bits where x is a normal double of
-// exponent field >= 3 (a subtraction on the integer pipes), else (zero, tiny,
-// infinite or NaN x) a multiplication, taken only in warps where a lane
-// needs it
-__device__ __forceinline__ double quarter_nonneg(double x) {
-  const long long b = dbits(x);
-  const bool fast = b >= (3LL << 52) && b < 0x7ff0000000000000LL;
-  double r = __longlong_as_double(b - (2LL << 52));
-  if (__any_sync(__activemask(), !fast)) {
-    if (!fast) r = 0.25 * x;
-  }
-  return r;
+// The energy that puts the pressure at its floor (t2 = m.v + |B_cc|^2).  A call,
+// made only in warps where a cell is floored: inlined, every warp issues its
+// FP64 instructions, two of the 14 to 20 of the primitive kernels.
+static __device__ __noinline__ double floored_energy(double p_floor, double igm1, double t2) {
+  return p_floor * igm1 + 0.5 * t2;
 }
 
 // FP32-bulk gas-pressure recovery in double: t2 = |m|^2 / rho' + |B_cc|^2
@@ -244,7 +265,7 @@ __device__ __forceinline__ void p_recover_f32(double ir, double m0, double m1, d
                                               double& t2, double& pe) {
   const double mm = fma(m0, m0, fma(m1, m1, m2 * m2));
   const double bb = fma(bsum[0], bsum[0], fma(bsum[1], bsum[1], bsum[2] * bsum[2]));
-  t2 = fma(mm, ir, quarter_nonneg(bb));
+  t2 = fma(mm, ir, quarter<double>(bb));
   pe = fma(-0.5, t2, e);
 }
 
@@ -274,6 +295,18 @@ __device__ __forceinline__ void prim_store_f32(const Grid& g, const Fields<float
   for (int f = 0; f < 8; ++f) W.f[f][c] = w8[f];
 }
 
+// end-of-step pressure floor of one cell (floors null: none); in: an interior cell
+__device__ __forceinline__ void floor_energy(const Grid& g, const Fields<double, 8>& U, int c,
+                                             unsigned long long* floors, bool in, double pg, double t2) {
+  const bool low = floors && lt_pos<double>(pg, g.p_floor);
+  if (__any_sync(__activemask(), low)) {
+    if (low) {
+      U.f[4][c] = floored_energy(g.p_floor, g.igm1, t2);
+      if (in) atomicAdd(&floors[1], 1ull);
+    }
+  }
+}
+
 // ------------------------------------------------------------------ Step 1 --
 // Primitives W of a state, and optionally (floors != nullptr) the end-of-step
 // floors of the conserved state (D-12): rho < rho_floor is raised; if the
@@ -284,7 +317,7 @@ __device__ __forceinline__ void prim_store_f32(const Grid& g, const Fields<float
 template <class T>
 __global__ void __launch_bounds__(BX* BY) k_prim(Grid g, Fields<double, 8> U, Fields<T, 8> W, unsigned long long* dtbits,
                                                  unsigned* flags, unsigned long long* floors, Fields<T, 3> Er) {
-  const Cell p = thread_cell(g);
+  const Cell p = step_cell(g);
   T inv = T(0);
   bool wd = false;  // (double, float pairs) this cell's primitives wk enter the CFL maximum
   double wr = 0.0, wp = 0.0;  // its density and pressure
@@ -315,19 +348,13 @@ __global__ void __launch_bounds__(BX* BY) k_prim(Grid g, Fields<double, 8> U, Fi
       double t2, pg;
       prim_store_f32(g, W, c, rho, ir, m0, m1, m2, e, bs, w8, t2, pg);
       store_ref<T>(Er, c, w8);
-      if (floors && lt_pos<double>(pg, g.p_floor)) {
-        U.f[4][c] = g.p_floor * g.igm1 + 0.5 * t2;
-        if (in) atomicAdd(&floors[1], 1ull);
-      }
+      floor_energy(g, U, c, floors, in, pg, t2);
       if (dtbits && in) inv = cell_inv_crossing<T>(g, w8);
     } else {
       const double b[3] = {half<double>(b0m + b0p), half<double>(b1m + b1p), half<double>(b2m + b2p)};
       double t2, pg;
       const PrimD pw = prim_core_ir(g, rho, ir, m0, m1, m2, e, b, t2, pg);
-      if (floors && lt_pos<double>(pg, g.p_floor)) {
-        U.f[4][c] = g.p_floor * g.igm1 + 0.5 * t2;
-        if (in) atomicAdd(&floors[1], 1ull);
-      }
+      floor_energy(g, U, c, floors, in, pg, t2);
       store_w<T>(W, c, pw, w8);
       store_ref<T>(Er, c, w8);
       if (dtbits && in) {
@@ -406,6 +433,10 @@ template <int A, class T> __device__ __forceinline__ void load_dir(const Fields<
   w[6] = ldg(W.f[5 + C] + q);
 }
 
+// blocks per SM of the Riemann kernels: the float-pair ones fit 80 registers
+// without spilling (6 blocks; 1.2 % faster than the allocator's own 96)
+template <class T> struct FluxMinBlocks { static constexpr int v = std::is_same<T, df>::value ? 6 : 0; };
+
 // -------------------------------------------------------------- Steps 2-3 --
 // one axis per launch: a thread solving three Riemann problems in sequence
 // holds too many registers for the occupancy the double-float arithmetic
@@ -423,9 +454,9 @@ __device__ __forceinline__ void flux_pcm_cell(const Grid& g, const Cell& p, cons
 }
 
 template <class T, int A>
-__global__ void __launch_bounds__(BX* BY) k_flux_pcm(Grid g, Fields<const T, 8> W, const double* __restrict__ BA,
+__global__ void __launch_bounds__(BX* BY, FluxMinBlocks<T>::v) k_flux_pcm(Grid g, Fields<const T, 8> W, const double* __restrict__ BA,
                                                      Fields<T, 7> FA) {
-  const Cell p = thread_cell(g);
+  const Cell p = step_cell(g);
   if (p.ok) flux_pcm_cell<T, A>(g, p, W, BA, FA.f);
 }
 
@@ -433,7 +464,7 @@ template <class T>
 __global__ void __launch_bounds__(BX* BY) k_flux_pcm3(Grid g, Fields<const T, 8> W, Fields<const double, 3> B,
                                                       Fields<T, 21> F) {
   const int a = block_axis(g);
-  const Cell p = thread_cell(g, blockIdx.z - a * g.n[2]);
+  const Cell p = step_cell(g, blockIdx.z - a * g.n[2]);
   if (!p.ok) return;
   if (a == 0) flux_pcm_cell<T, 0>(g, p, W, B.f[0], F.f);
   else if (a == 1) flux_pcm_cell<T, 1>(g, p, W, B.f[1], F.f + 7);
@@ -446,16 +477,12 @@ template <class T> __device__ __forceinline__ void floor_face(const Grid& g, T* 
   w[4] = max_pos<T>(w[4], from_d<T>(g.p_floor));
 }
 
-// blocks of 128 threads per SM requested from the register allocator.  4 (at
-// most 128 registers per thread) for float pairs and float: the float-pair
-// kernels lose 9 % (PPMC) and 12 % (PLMC) at 3 blocks, their dependent chains
-// need the extra warps.  3 (168 registers) for the double PLMC and PPMC
-// kernels, which interleave integer-pipe products with the FP64 pipe: at 4
-// blocks they spill 0.5 KB (256^3: 22.4 and 40.6 ms against 21.4 and 38.6 ms).
-template <class T, int RECON> struct ReconMinBlocks {
-  static constexpr int v = std::is_same<T, double>::value && (RECON == 1 || RECON == 2) ? 3 : 4;
-};
-
+// blocks of 128 threads per SM requested from the register allocator: 4 (at
+// most 128 registers per thread).  The float-pair kernels lose 9 % (PPMC) and
+// 12 % (PLMC) at 3 blocks, their dependent chains need the extra warps, and 7 %
+// and 1 % at 5 (spills); the double ones, which spill 0.2 KB at 4, lose 6 % and
+// 9 % at 3.
+template <class T, int RECON> struct ReconMinBlocks { static constexpr int v = 4; };
 // interface states of cell p along A (Step 6): wl = W_{L,i+1/2} (the cell's
 // state at its upper face), wr = W_{R,i-1/2} (at its lower face), floored
 template <class T, int RECON, int A, class O>
@@ -490,7 +517,7 @@ __device__ __noinline__ void recon_cell_again(const Grid& g, const Fields<const 
 }
 template <class T, int RECON, int A>
 __device__ __forceinline__ void recon_cell(const Grid& g, const Fields<const T, 8>& W, const Cell& p, T* wl, T* wr) {
-  TryOps<T> o;
+  CallOps<T> o;
   recon_cell_with<T, RECON, A>(o, g, W, p, wl, wr);
   if constexpr (std::is_same<T, double>::value && (RECON == 1 || RECON == 2)) {
     if (__any_sync(__activemask(), o.bad)) {
@@ -511,7 +538,7 @@ __device__ __forceinline__ void recon_cell(const Grid& g, const Fields<const T, 
 template <class T, int RECON, int A>
 __global__ void __launch_bounds__(BX* BY, ReconMinBlocks<T, RECON>::v) k_recon(Grid g, Fields<const T, 8> W,
                                                                              Fields<T, 7> WL, Fields<T, 7> WR) {
-  const Cell p = thread_cell(g);
+  const Cell p = step_cell(g);
   if (!p.ok) return;
   T wl[7], wr[7];
   recon_cell<T, RECON, A>(g, W, p, wl, wr);
@@ -537,7 +564,7 @@ template <class T, int RECON>
 __global__ void __launch_bounds__(BX* BY, ReconMinBlocks<T, RECON>::v) k_recon3(Grid g, Fields<const T, 8> W,
                                                                               Fields<T, 21> WL, Fields<T, 21> WR) {
   const int a = block_axis(g);
-  const Cell p = thread_cell(g, blockIdx.z - a * g.n[2]);
+  const Cell p = step_cell(g, blockIdx.z - a * g.n[2]);
   if (!p.ok) return;
   if (a == 0) recon_axis<T, RECON, 0>(g, W, p, WL, WR);
   else if (a == 1) recon_axis<T, RECON, 1>(g, W, p, WL, WR);
@@ -562,9 +589,9 @@ __device__ __forceinline__ void flux_hlld_cell(const Grid& g, const Cell& p, con
 }
 
 template <class T, int A>
-__global__ void __launch_bounds__(BX* BY) k_flux_hlld(Grid g, Fields<const T, 7> WL, Fields<const T, 7> WR,
+__global__ void __launch_bounds__(BX* BY, FluxMinBlocks<T>::v) k_flux_hlld(Grid g, Fields<const T, 7> WL, Fields<const T, 7> WR,
                                                       const T* __restrict__ BfA, Fields<T, 7> FA) {
-  const Cell p = thread_cell(g);
+  const Cell p = step_cell(g);
   if (p.ok) flux_hlld_cell<T, A>(g, p, WL.f, WR.f, BfA, FA.f);
 }
 
@@ -572,7 +599,7 @@ template <class T>
 __global__ void __launch_bounds__(BX* BY) k_flux_hlld3(Grid g, Fields<const T, 21> WL, Fields<const T, 21> WR,
                                                        Fields<const T, 3> Bf, Fields<T, 21> F) {
   const int a = block_axis(g);
-  const Cell p = thread_cell(g, blockIdx.z - a * g.n[2]);
+  const Cell p = step_cell(g, blockIdx.z - a * g.n[2]);
   if (!p.ok) return;
   if (a == 0) flux_hlld_cell<T, 0>(g, p, WL.f, WR.f, Bf.f[0], F.f);
   else if (a == 1) flux_hlld_cell<T, 1>(g, p, WL.f + 7, WR.f + 7, Bf.f[1], F.f + 7);
@@ -587,7 +614,7 @@ __global__ void __launch_bounds__(BX* BY) k_flux_hlld3(Grid g, Fields<const T, 2
 template <class T, int A>
 __global__ void __launch_bounds__(BX* BY) k_flux_hlld_r(Grid g, const T* __restrict__ WL, const T* __restrict__ WR,
                                                         const T* __restrict__ Bf, T* __restrict__ F) {
-  const CellIdx ci = cell_of_thread(g);
+  const CellIdx ci = step_cell_idx(g);
   if (!ci.ok) return;
   const long long N = g.N, c = cidx(g, ci.i, ci.j, ci.k), cn = nb<A>(g, ci.i, ci.j, ci.k, 1);
   T wl[7], wr[7], f[7];
@@ -697,7 +724,7 @@ __device__ __forceinline__ T edge_field(const Grid& g, const Fields<const T, 8>&
 template <class T, bool REF>
 __global__ void __launch_bounds__(BX* BY) k_emf(Grid g, Fields<const T, 8> W, Fields<const T, 21> F,
                                                 Fields<const T, 3> Er, Fields<T, 3> E) {
-  const Cell p = thread_cell(g);
+  const Cell p = step_cell(g);
   if (!p.ok) return;
   const T e0 = edge_field<T, 0, REF>(g, W, F, Er, p);
   const T e1 = edge_field<T, 1, REF>(g, W, F, Er, p);
@@ -742,7 +769,7 @@ __device__ __forceinline__ T edge_field_r(const Grid& g, const T* __restrict__ W
 template <class T, bool REF>
 __global__ void __launch_bounds__(BX* BY) k_emf_r(Grid g, const T* __restrict__ W, const T* __restrict__ F,
                                                   const T* __restrict__ Er, T* __restrict__ E) {
-  const CellIdx ci = cell_of_thread(g);
+  const CellIdx ci = step_cell_idx(g);
   if (!ci.ok) return;
   const long long N = g.N, c = cidx(g, ci.i, ci.j, ci.k);
   E[c] = edge_field_r<T, 0, REF>(g, W, F, Er, ci.i, ci.j, ci.k);
@@ -863,7 +890,7 @@ __global__ void __launch_bounds__(BX* BY) k_update_half(Grid g, Fields<const dou
                                                         Fields<const T, 3> E, const double* __restrict__ dtp,
                                                         Fields<T, 8> W, Fields<T, 3> Bh, unsigned* flags,
                                                         Fields<T, 3> Er) {
-  const Cell p = thread_cell(g);
+  const Cell p = step_cell(g);
   if (!p.ok) return;
   const int c = p.c;
   const StepScalars& S = *reinterpret_cast<const StepScalars*>(dtp);
@@ -904,7 +931,7 @@ __global__ void __launch_bounds__(BX* BY) k_update_half(Grid g, Fields<const dou
 template <class T>
 __global__ void __launch_bounds__(BX* BY) k_update_full(Grid g, Fields<double, 8> U, Fields<const T, 21> F,
                                                         Fields<const T, 3> E, const double* __restrict__ dtp) {
-  const Cell p = thread_cell(g);
+  const Cell p = step_cell(g);
   if (!p.ok) return;
   const int c = p.c;
   const StepScalars& S = *reinterpret_cast<const StepScalars*>(dtp);
@@ -962,6 +989,7 @@ __global__ void k_set_dt(Grid g, double* dt_cur, double value) {
 // past t_end (t_end = +inf: no end time); the shortened step lands on t_end.
 __global__ void k_finish_dt(Grid g, unsigned long long* dtbits, double* dt_cur, double* dt_log, int s,
                             unsigned* flags, double t_end) {
+  grid_wait(s);
   const double m = __longlong_as_double((long long)dtbits[0]);
   double dt = g.cfl / m;
   if (!(dt > 0.0) || !isfinite(dt)) atomicOr(flags, 2u);
@@ -1156,29 +1184,45 @@ __global__ void __launch_bounds__(DIAG_T) k_diag_final(const double* red_in, dou
 
 // --------------------------------------------------------------- launchers --
 
+// one step kernel on stream s, launched early (grid_wait)
+template <class... P, class... A>
+static void launch_step(void (*k)(P...), dim3 grid, cudaStream_t s, const A&... args) {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3(BX, BY);
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, k, P(args)...);
+}
+
 template <class T>
 void Launch<T>::prim(const Grid& g, double* U, T* W, unsigned long long* dtbits, unsigned* flags,
                      unsigned long long* floors, cudaStream_t s, T* Er) {
+  // (not early: it may follow k_update_full)
   k_prim<T><<<grid_of(g), dim3(BX, BY), 0, s>>>(g, fields<8>(U, g.N), fields<8>(W, g.N), dtbits, flags, floors,
                                                 fields<3>(Er, g.N));
 }
 template <class T>
 void Launch<T>::flux_pcm(const Grid& g, int a, const T* W, const double* U, T* F, cudaStream_t s) {
-  const dim3 gr = grid_of(g), bl(BX, BY);
+  const dim3 gr = grid_of(g);
   const Fields<const T, 8> Wf = fields<8>(W, g.N);
   const Fields<T, 7> Fa = fields<7>(F + a * 7 * g.N, g.N);
   const double* Ba = U + (5 + a) * g.N;
-  if (a == 0) k_flux_pcm<T, 0><<<gr, bl, 0, s>>>(g, Wf, Ba, Fa);
-  if (a == 1) k_flux_pcm<T, 1><<<gr, bl, 0, s>>>(g, Wf, Ba, Fa);
-  if (a == 2) k_flux_pcm<T, 2><<<gr, bl, 0, s>>>(g, Wf, Ba, Fa);
+  if (a == 0) launch_step(k_flux_pcm<T, 0>, gr, s, g, Wf, Ba, Fa);
+  if (a == 1) launch_step(k_flux_pcm<T, 1>, gr, s, g, Wf, Ba, Fa);
+  if (a == 2) launch_step(k_flux_pcm<T, 2>, gr, s, g, Wf, Ba, Fa);
 }
 template <class T, int RC>
 static void launch_recon(const Grid& g, int a, const Fields<const T, 8>& W, const Fields<T, 7>& WL,
                          const Fields<T, 7>& WR, cudaStream_t s) {
-  const dim3 gr = grid_of(g), bl(BX, BY);
-  if (a == 0) k_recon<T, RC, 0><<<gr, bl, 0, s>>>(g, W, WL, WR);
-  if (a == 1) k_recon<T, RC, 1><<<gr, bl, 0, s>>>(g, W, WL, WR);
-  if (a == 2) k_recon<T, RC, 2><<<gr, bl, 0, s>>>(g, W, WL, WR);
+  const dim3 gr = grid_of(g);
+  if (a == 0) launch_step(k_recon<T, RC, 0>, gr, s, g, W, WL, WR);
+  if (a == 1) launch_step(k_recon<T, RC, 1>, gr, s, g, W, WL, WR);
+  if (a == 2) launch_step(k_recon<T, RC, 2>, gr, s, g, W, WL, WR);
 }
 template <class T>
 void Launch<T>::recon(const Grid& g, int rc, int a, const T* W, T* WL, T* WR, cudaStream_t s) {
@@ -1191,64 +1235,64 @@ void Launch<T>::recon(const Grid& g, int rc, int a, const T* W, T* WL, T* WR, cu
 }
 template <class T>
 void Launch<T>::flux_pcm3(const Grid& g, const T* W, const double* U, T* F, cudaStream_t s) {
-  k_flux_pcm3<T><<<grid3_of(g), dim3(BX, BY), 0, s>>>(g, fields<8>(W, g.N), fields<3>(U + 5 * g.N, g.N),
+  launch_step(k_flux_pcm3<T>, grid3_of(g), s, g, fields<8>(W, g.N), fields<3>(U + 5 * g.N, g.N),
                                                       fields<21>(F, g.N));
 }
 template <class T>
 void Launch<T>::recon3(const Grid& g, int rc, const T* W, T* WL, T* WR, cudaStream_t s) {
   const Fields<const T, 8> Wf = fields<8>(W, g.N);
   const Fields<T, 21> L = fields<21>(WL, g.N), R = fields<21>(WR, g.N);
-  const dim3 gr = grid3_of(g), bl(BX, BY);
-  if (rc == 0) k_recon3<T, 0><<<gr, bl, 0, s>>>(g, Wf, L, R);
-  else if (rc == 1) k_recon3<T, 1><<<gr, bl, 0, s>>>(g, Wf, L, R);
-  else if (rc == 2) k_recon3<T, 2><<<gr, bl, 0, s>>>(g, Wf, L, R);
-  else k_recon3<T, 3><<<gr, bl, 0, s>>>(g, Wf, L, R);
+  const dim3 gr = grid3_of(g);
+  if (rc == 0) launch_step(k_recon3<T, 0>, gr, s, g, Wf, L, R);
+  else if (rc == 1) launch_step(k_recon3<T, 1>, gr, s, g, Wf, L, R);
+  else if (rc == 2) launch_step(k_recon3<T, 2>, gr, s, g, Wf, L, R);
+  else launch_step(k_recon3<T, 3>, gr, s, g, Wf, L, R);
 }
 template <class T>
 void Launch<T>::flux_hlld3(const Grid& g, const T* WL, const T* WR, const T* Bf, T* F, cudaStream_t s) {
-  k_flux_hlld3<T><<<grid3_of(g), dim3(BX, BY), 0, s>>>(g, fields<21>(WL, g.N), fields<21>(WR, g.N),
+  launch_step(k_flux_hlld3<T>, grid3_of(g), s, g, fields<21>(WL, g.N), fields<21>(WR, g.N),
                                                        fields<3>(Bf, g.N), fields<21>(F, g.N));
 }
 template <class T>
 void Launch<T>::flux_hlld(const Grid& g, int a, const T* WL, const T* WR, const T* Bf, T* F, cudaStream_t s) {
-  const dim3 gr = grid_of(g), bl(BX, BY);
+  const dim3 gr = grid_of(g);
   if constexpr (std::is_same<T, float>::value) {
-    if (a == 0) k_flux_hlld_r<T, 0><<<gr, bl, 0, s>>>(g, WL, WR, Bf, F);
-    if (a == 1) k_flux_hlld_r<T, 1><<<gr, bl, 0, s>>>(g, WL, WR, Bf, F);
-    if (a == 2) k_flux_hlld_r<T, 2><<<gr, bl, 0, s>>>(g, WL, WR, Bf, F);
+    if (a == 0) launch_step(k_flux_hlld_r<T, 0>, gr, s, g, WL, WR, Bf, F);
+    if (a == 1) launch_step(k_flux_hlld_r<T, 1>, gr, s, g, WL, WR, Bf, F);
+    if (a == 2) launch_step(k_flux_hlld_r<T, 2>, gr, s, g, WL, WR, Bf, F);
     return;
   }
   const Fields<const T, 7> L = fields<7>(WL, g.N), R = fields<7>(WR, g.N);
   const Fields<T, 7> Fa = fields<7>(F + a * 7 * g.N, g.N);
   const T* Ba = Bf + a * g.N;
-  if (a == 0) k_flux_hlld<T, 0><<<gr, bl, 0, s>>>(g, L, R, Ba, Fa);
-  if (a == 1) k_flux_hlld<T, 1><<<gr, bl, 0, s>>>(g, L, R, Ba, Fa);
-  if (a == 2) k_flux_hlld<T, 2><<<gr, bl, 0, s>>>(g, L, R, Ba, Fa);
+  if (a == 0) launch_step(k_flux_hlld<T, 0>, gr, s, g, L, R, Ba, Fa);
+  if (a == 1) launch_step(k_flux_hlld<T, 1>, gr, s, g, L, R, Ba, Fa);
+  if (a == 2) launch_step(k_flux_hlld<T, 2>, gr, s, g, L, R, Ba, Fa);
 }
 template <class T>
 void Launch<T>::emf(const Grid& g, const T* W, const T* F, T* E, cudaStream_t s, const T* Er) {
   if constexpr (std::is_same<T, double>::value) {
-    if (Er) k_emf_r<T, true><<<grid_of(g), dim3(BX, BY), 0, s>>>(g, W, F, Er, E);
-    else k_emf_r<T, false><<<grid_of(g), dim3(BX, BY), 0, s>>>(g, W, F, Er, E);
+    if (Er) launch_step(k_emf_r<T, true>, grid_of(g), s, g, W, F, Er, E);
+    else launch_step(k_emf_r<T, false>, grid_of(g), s, g, W, F, Er, E);
     return;
   }
   const Fields<const T, 8> Wf = fields<8>(W, g.N);
   const Fields<const T, 21> Ff = fields<21>(F, g.N);
   const Fields<const T, 3> Rf = fields<3>(Er, g.N);
   const Fields<T, 3> Ef = fields<3>(E, g.N);
-  if (Er) k_emf<T, true><<<grid_of(g), dim3(BX, BY), 0, s>>>(g, Wf, Ff, Rf, Ef);
-  else k_emf<T, false><<<grid_of(g), dim3(BX, BY), 0, s>>>(g, Wf, Ff, Rf, Ef);
+  if (Er) launch_step(k_emf<T, true>, grid_of(g), s, g, Wf, Ff, Rf, Ef);
+  else launch_step(k_emf<T, false>, grid_of(g), s, g, Wf, Ff, Rf, Ef);
 }
 template <class T>
 void Launch<T>::update_half(const Grid& g, const double* U, const T* F, const T* E, const double* dtp, T* W, T* Bh,
                             unsigned* flags, cudaStream_t s, T* Er) {
-  k_update_half<T><<<grid_of(g), dim3(BX, BY), 0, s>>>(g, fields<8>(U, g.N), fields<21>(F, g.N), fields<3>(E, g.N),
+  launch_step(k_update_half<T>, grid_of(g), s, g, fields<8>(U, g.N), fields<21>(F, g.N), fields<3>(E, g.N),
                                                        dtp, fields<8>(W, g.N), fields<3>(Bh, g.N), flags,
                                                        fields<3>(Er, g.N));
 }
 template <class T>
 void Launch<T>::update_full(const Grid& g, double* U, const T* F, const T* E, const double* dtp, cudaStream_t s) {
-  k_update_full<T><<<grid_of(g), dim3(BX, BY), 0, s>>>(g, fields<8>(U, g.N), fields<21>(F, g.N), fields<3>(E, g.N),
+  launch_step(k_update_full<T>, grid_of(g), s, g, fields<8>(U, g.N), fields<21>(F, g.N), fields<3>(E, g.N),
                                                        dtp);
 }
 template <class T>
