@@ -285,6 +285,11 @@ def roofline_of(prof, precision, n3, hbm_peak, peak_kind, recon="plmc"):
     """
     T = 4 if precision == "fp32_bulk" else 8
     sb = stage_bytes(T)
+    # (grids of up to 128^3 run the three axes of a stage as one launch; bytes
+    # and counters are those of one axis)
+    n_steps = max(1, prof["update_full"][1])
+    prof = {k: (v[0], 3 * n_steps) if k in ("flux_pcm", "recon", "flux_hlld") and v[1] == n_steps else v
+            for k, v in prof.items()}
     total = sum(v[0] for v in prof.values())
     name, (ms, launches) = max(prof.items(), key=lambda kv: kv[1][0])
     per_launch_s = ms / max(launches, 1) * 1e-3

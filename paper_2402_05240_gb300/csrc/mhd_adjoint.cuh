@@ -55,13 +55,8 @@ template <class T> struct EigCoefG {
   __device__ void zero() { fp = sp = fb = sb = fu = su = z1 = z2 = T(0); }
 };
 template <class T>
-__device__ __forceinline__ void eig_left_vjp_wide(const Eig<T>& E, const T* dw, const T* gq, T* gdw, EigG<T>& gE,
-                                                  EigCoefG<T>& gC) {
-  const T n = half<T>(E.ia2);
-  const T naf = n * E.af, nas = n * E.as, ai = E.a * E.isr;
-  const T fp = naf * E.ir, sp = nas * E.ir, fb = nas * ai, sb = naf * ai, fu = naf * E.cf, su = nas * E.cs;
-  const T z = half<T>(times_sign<T>(E.isr, E.sg));
-  const T z1 = E.b1 * z, z2 = E.b2 * z;
+__device__ __forceinline__ void eig_left_vjp_wide(const Eig<T>& E, const EigCoef<T>& C, const T* dw, const T* gq,
+                                                  T* gdw, EigG<T>& gE, EigCoefG<T>& gC) {
   const T bv = times_sign<T>(E.b1 * dw[2] + E.b2 * dw[3], E.sg);
   const T bb = E.b1 * dw[5] + E.b2 * dw[6];
   const T gXf = gq[0] + gq[6], gYf = gq[0] - gq[6];
@@ -75,18 +70,18 @@ __device__ __forceinline__ void eig_left_vjp_wide(const Eig<T>& E, const T* dw, 
   gC.fu += gYs * bv - gYf * dw[1];
   gC.z1 += gZb * dw[6];
   gC.z2 -= gZb * dw[5];
-  const T gbb = gXf * fb - gXs * sb;
-  const T gbv = times_sign<T>(gYf * su + gYs * fu, E.sg);
+  const T gbb = gXf * C.fb - gXs * C.sb;
+  const T gbv = times_sign<T>(gYf * C.su + gYs * C.fu, E.sg);
   gE.ia2 -= gq[3] * dw[4];
   gE.b1 += gbv * dw[2] + gbb * dw[5] + hZ * dw[3];
   gE.b2 += gbv * dw[3] + gbb * dw[6] - hZ * dw[2];
   gdw[0] = gq[3];
-  gdw[1] = gYs * su - gYf * fu;
+  gdw[1] = gYs * C.su - gYf * C.fu;
   gdw[2] = gbv * E.b1 - hZ * E.b2;
   gdw[3] = gbv * E.b2 + hZ * E.b1;
-  gdw[4] = gXf * fp + gXs * sp - gq[3] * E.ia2;
-  gdw[5] = gbb * E.b1 - gZb * z2;
-  gdw[6] = gbb * E.b2 + gZb * z1;
+  gdw[4] = gXf * C.fp + gXs * C.sp - gq[3] * E.ia2;
+  gdw[5] = gbb * E.b1 - gZb * C.z2;
+  gdw[6] = gbb * E.b2 + gZb * C.z1;
 }
 template <class T> __device__ __forceinline__ void eig_coef_vjp(const Eig<T>& E, const EigCoefG<T>& gC, EigG<T>& gE) {
   if constexpr (sizeof(T) == 4) return;
@@ -252,22 +247,22 @@ __device__ __forceinline__ void eig_fields_vjp(T gamma, const T* w0, T bn, const
   // forward values: the roots and reciprocals come from the forward
   // eigensystem E of the same state (eig_build), the rest is recomputed
   const T ir = E.ir, a2 = E.a2, ia2 = E.ia2, cf = E.cf, cs = E.cs, sr = E.sr, isr = E.isr, a = E.a;
-  const T ca2 = bn * bn * ir;
+  const T ca2 = mulc<T>(mulc<T>(bn, bn), ir);
   const T bt2r = by * by + bz * bz;
-  const T bt2 = bt2r * ir;
+  const T bt2 = mulc<T>(bt2r, ir);
   const T b2 = ca2 + bt2;
   const T D = a2 - b2;
-  const T sd = tsqrt<T>(D * D + quad<T>(a2) * bt2);
-  const T icf2 = E.rcf * E.rcf;
-  const T cs2 = a2 * ca2 * icf2;
+  const T sd = tsqrt<T>(D * D + mulc<T>(quad<T>(a2), bt2));
+  const T icf2 = mulc<T>(E.rcf, E.rcf);
+  const T cs2 = mulc<T>(mulc<T>(a2, ca2), icf2);
   const T sg = E.sg;
   // magnetosonic normalisations: af = sqrt(uf), as = sqrt(us)
   const int br = is0<T>(sd) ? 0 : (ge0<T>(D) ? 1 : 2);
   const T af = E.af, as = E.as;
   T M = T(0), N = T(0), iM = T(0), r2s = T(0);
   if (br != 0) {
-    N = twice<T>(a2) * bt2;
-    M = br == 1 ? sd * (sd + D) : sd * (sd - D);
+    N = mulc<T>(twice<T>(a2), bt2);
+    M = mulc<T>(sd, br == 1 ? T(sd + D) : T(sd - D));
     iM = trcp<T>(M);
     r2s = trcp<T>(twice<T>(sd));
   }
@@ -311,8 +306,8 @@ __device__ __forceinline__ void eig_fields_vjp(T gamma, const T* w0, T bn, const
     // d big / d sd = -sD D / (2 sd^2), d big / d D = sD / (2 sd)
     g_sd += -g_big * sD * D * r2s * r2s * T(2);
     g_D += g_big * sD * r2s;
-    const T g_N = g_small * iM;
-    const T g_M = -g_small * N * iM * iM;
+    const T g_N = mulc<T>(g_small, iM);
+    const T g_M = -mulc<T>(mulc<T>(mulc<T>(g_small, N), iM), iM);
     g_a2 += twice<T>(g_N) * bt2;
     g_bt2 += twice<T>(g_N) * a2;
     // M = sd (sd + sD D)
@@ -330,7 +325,7 @@ __device__ __forceinline__ void eig_fields_vjp(T gamma, const T* w0, T bn, const
   g_sd += T(0.5) * g_cf2;
   // sd = sqrt(D^2 + 4 a2 bt2)
   if (sd > T(0)) {
-    const T g_X = g_sd * r2s;  // (sd > 0: r2s = 1/(2 sd))
+    const T g_X = mulc<T>(g_sd, r2s);  // (sd > 0: r2s = 1/(2 sd))
     g_D += twice<T>(g_X) * D;
     g_a2 += quad<T>(g_X) * bt2;
     g_bt2 += quad<T>(g_X) * a2;
@@ -367,11 +362,13 @@ __device__ __forceinline__ void eig_fields_vjp(T gamma, const T* w0, T bn, const
 template <class T> struct OutlineRev { static constexpr bool v = false; };
 template <> struct OutlineRev<df> { static constexpr bool v = true; };
 template <class T>
-__device__ __noinline__ void eig_left_vjp_call(const Eig<T>& E, const T* dw, const T* gq, T* gdw, EigG<T>& gE,
-                                               EigCoefG<T>& gC) {
-  eig_left_vjp_wide<T>(E, dw, gq, gdw, gE, gC);
+__device__ __noinline__ void eig_left_vjp_call(const Eig<T>& E, const EigCoef<T>& C, const T* dw, const T* gq, T* gdw,
+                                               EigG<T>& gE, EigCoefG<T>& gC) {
+  eig_left_vjp_wide<T>(E, C, dw, gq, gdw, gE, gC);
 }
-template <class T> __device__ __noinline__ void eig_left_call(const Eig<T>& E, const T* dw, T* q) { eig_left<T>(E, dw, q); }
+template <class T> __device__ __noinline__ void eig_left_call(const Eig<T>& E, const EigCoef<T>& C, const T* dw, T* q) {
+  eig_left<T>(E, C, dw, q);
+}
 template <class T>
 __device__ __noinline__ void eig_right_vjp_call(const Eig<T>& E, const T* q, const T* gdw, T* gq, EigG<T>& gE) {
   eig_right_vjp<T>(E, q, gdw, gq, gE);
@@ -386,16 +383,16 @@ template <class T> __device__ __forceinline__ void ppm_one_o(const T* col, T& qm
     ppm_one<T>(col, qm, qp);
   }
 }
-template <class T> __device__ __forceinline__ void eig_left_o(const Eig<T>& E, const T* dw, T* q) {
-  if constexpr (OutlineRev<T>::v) eig_left_call<T>(E, dw, q);
-  else eig_left<T>(E, dw, q);
+template <class T> __device__ __forceinline__ void eig_left_o(const Eig<T>& E, const EigCoef<T>& C, const T* dw, T* q) {
+  if constexpr (OutlineRev<T>::v) eig_left_call<T>(E, C, dw, q);
+  else eig_left<T>(E, C, dw, q);
 }
 // (gdw zero on entry)
 template <class T>
-__device__ __forceinline__ void eig_left_vjp_o(const Eig<T>& E, T ir, const T* dw, const T* gq, T* gdw, EigG<T>& gE,
-                                               EigCoefG<T>& gC) {
-  if constexpr (OutlineRev<T>::v) eig_left_vjp_call<T>(E, dw, gq, gdw, gE, gC);
-  else if constexpr (sizeof(T) != 4) eig_left_vjp_wide<T>(E, dw, gq, gdw, gE, gC);
+__device__ __forceinline__ void eig_left_vjp_o(const Eig<T>& E, const EigCoef<T>& C, T ir, const T* dw, const T* gq,
+                                               T* gdw, EigG<T>& gE, EigCoefG<T>& gC) {
+  if constexpr (OutlineRev<T>::v) eig_left_vjp_call<T>(E, C, dw, gq, gdw, gE, gC);
+  else if constexpr (sizeof(T) != 4) eig_left_vjp_wide<T>(E, C, dw, gq, gdw, gE, gC);
   else eig_left_vjp<T>(E, ir, dw, gq, gdw, gE);
 }
 template <class T>
@@ -419,11 +416,13 @@ __device__ void plmc_vjp(T gamma, T rho_floor, T p_floor, const T* wm, const T* 
   van_leer7<T>(dL, dR, dG);  // the forward's arithmetic (plmc)
   Eig<T> E;
   eig_build<T>(gamma, w0, bn, E);
+  Ops<T> ops;
+  const EigCoef<T> C = eig_coef<T>(ops, E);
   const T ir = E.ir;
   T aL[7], aR[7], aC[7], aG[7], am[7], dW[7];
-  eig_left_o<T>(E, dL, aL);
-  eig_left_o<T>(E, dR, aR);
-  eig_left_o<T>(E, dG, aG);
+  eig_left_o<T>(E, C, dL, aL);
+  eig_left_o<T>(E, C, dR, aR);
+  eig_left_o<T>(E, C, dG, aG);
 #pragma unroll
   for (int q = 0; q < 7; ++q) aC[q] = T(0.5) * (aL[q] + aR[q]);
   int sel[7];  // -1: zero slope; 0..3: candidate 2|aL|, 2|aR|, |aC|, |aG|
@@ -488,9 +487,9 @@ __device__ void plmc_vjp(T gamma, T rho_floor, T p_floor, const T* wm, const T* 
   }
   EigCoefG<T> gC;
   gC.zero();
-  eig_left_vjp_o<T>(E, ir, dL, gaL, gdL, gE, gC);
-  eig_left_vjp_o<T>(E, ir, dR, gaR, gdR, gE, gC);
-  eig_left_vjp_o<T>(E, ir, dG, gaG, gdG, gE, gC);
+  eig_left_vjp_o<T>(E, C, ir, dL, gaL, gdL, gE, gC);
+  eig_left_vjp_o<T>(E, C, ir, dR, gaR, gdR, gE, gC);
+  eig_left_vjp_o<T>(E, C, ir, dG, gaG, gdG, gE, gC);
   eig_coef_vjp<T>(E, gC, gE);
 #pragma unroll
   for (int q = 0; q < 7; ++q) {
@@ -799,6 +798,8 @@ __device__ void ppmc_vjp(T gamma, T rho_floor, T p_floor, Load wload, T bn, cons
   wload(2, w2);
   Eig<T> E;
   eig_build<T>(gamma, w2, bn, E);
+  Ops<T> ops;
+  const EigCoef<T> C = eig_coef<T>(ops, E);
   const T ir = E.ir;
   T qs[4][7];  // deviations of cells i-2, i-1, i+1, i+2 (q of cell i is 0)
 #pragma unroll
@@ -807,7 +808,7 @@ __device__ void ppmc_vjp(T gamma, T rho_floor, T p_floor, Load wload, T bn, cons
     wload(k < 2 ? k : k + 1, wm);
 #pragma unroll
     for (int c = 0; c < 7; ++c) d[c] = wm[c] - w2[c];
-    eig_left_o<T>(E, d, qs[k]);
+    eig_left_o<T>(E, C, d, qs[k]);
   }
   T dm[7], dp[7];
 #pragma unroll
@@ -862,7 +863,7 @@ __device__ void ppmc_vjp(T gamma, T rho_floor, T p_floor, Load wload, T bn, cons
 #pragma unroll
     for (int c = 0; c < 7; ++c) d[c] = wm[c] - w2[c];
     T gd[7] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-    eig_left_vjp_o<T>(E, ir, d, gqs[k], gd, gE, gC);
+    eig_left_vjp_o<T>(E, C, ir, d, gqs[k], gd, gE, gC);
     put(k < 2 ? k : k + 1, gd);
 #pragma unroll
     for (int c = 0; c < 7; ++c) gw2[c] -= gd[c];
@@ -888,13 +889,15 @@ template <class T, class Load>
 __device__ __forceinline__ void ppmc_deviations(T gamma, Load wload, T bn, T* w2, Eig<T>& E, T (*qs)[7]) {
   wload(2, w2);
   eig_build<T>(gamma, w2, bn, E);
+  Ops<T> ops;
+  const EigCoef<T> C = eig_coef<T>(ops, E);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     T wm[7], d[7];
     wload(k < 2 ? k : k + 1, wm);
 #pragma unroll
     for (int c = 0; c < 7; ++c) d[c] = wm[c] - w2[c];
-    eig_left_o<T>(E, d, qs[k]);
+    eig_left_o<T>(E, C, d, qs[k]);
   }
 }
 
@@ -964,6 +967,8 @@ __device__ void ppmc_vjp_pass3(T gamma, Load wload, T bn, GqLoad gqload, EigG<T>
   wload(2, w2);
   Eig<T> E;
   eig_build<T>(gamma, w2, bn, E);
+  Ops<T> ops;
+  const EigCoef<T> C = eig_coef<T>(ops, E);
   const T ir = E.ir;
   EigCoefG<T> gC;
   gC.zero();
@@ -975,7 +980,7 @@ __device__ void ppmc_vjp_pass3(T gamma, Load wload, T bn, GqLoad gqload, EigG<T>
     for (int c = 0; c < 7; ++c) d[c] = wm[c] - w2[c];
     gqload(k, gq);
     T gd[7] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-    eig_left_vjp_o<T>(E, ir, d, gq, gd, gE, gC);
+    eig_left_vjp_o<T>(E, C, ir, d, gq, gd, gE, gC);
     put(k < 2 ? k : k + 1, gd);
 #pragma unroll
     for (int c = 0; c < 7; ++c) gw2[c] -= gd[c];
@@ -1101,32 +1106,32 @@ template <class T>
 __device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, const T* wr, T bn, const T* gf, T* gwl,
                                               T* gwr, T& gbn) {
   // forward (hlld_diff)
-  const T bn2 = bn * bn;
+  const T bn2 = mulc<T>(bn, bn);
   const T btL = wl[5] * wl[5] + wl[6] * wl[6], btR = wr[5] * wr[5] + wr[6] * wr[6];
   const T bbL = bn2 + btL, bbR = bn2 + btR;
   const T ptL = wl[4] + half<T>(bbL), ptR = wr[4] + half<T>(bbR);
   auto root = [&](T p, T bb, T bt) -> T {
-    const T gp = gamma * p;
+    const T gp = mulc<T>(gamma, p);
     const T dd = gp - bb;
-    return tsqrt<T>(dd * dd + quad<T>(gp) * bt);
+    return tsqrt<T>(dd * dd + mulc<T>(quad<T>(gp), bt));
   };
   const T sL = root(wl[4], bbL, btL), sR = root(wr[4], bbR, btR);
   const T XL = gamma * wl[4] + bbL + sL, XR = gamma * wr[4] + bbR + sR;
-  const bool lmax = !nonneg_lt<T>(XL * wr[0], XR * wl[0]);
+  const bool lmax = !nonneg_lt<T>(mulc<T>(XL, wr[0]), mulc<T>(XR, wl[0]));
   const T irc = trcp<T>(lmax ? wl[0] : wr[0]);
-  const T c2 = half<T>(lmax ? XL : XR) * irc;
+  const T c2 = mulc<T>(half<T>(lmax ? XL : XR), irc);
   const T cmax = tsqrt<T>(c2);
   const T SL = min_s<T>(wl[1], wr[1]) - cmax;
   const T SR = max_s<T>(wl[1], wr[1]) + cmax;
   const bool sub = !ge0<T>(SL) && !le0<T>(SR);
   T rdL = T(0), rdR = T(0), dlL = T(0), dlR = T(0), SM = T(0), pts = T(0), iden = T(0);
   if (sub) {
-    rdL = wl[0] * (SL - wl[1]);
-    rdR = wr[0] * (SR - wr[1]);
+    rdL = mulc<T>(wl[0], SL - wl[1]);
+    rdR = mulc<T>(wr[0], SR - wr[1]);
     iden = trcp<T>(rdR - rdL);
     const T du = wr[1] - wl[1], dp = ptL - ptR;
-    dlL = (rdR * du + dp) * iden;
-    dlR = (rdL * du + dp) * iden;
+    dlL = mulc<T>(rdR * du + dp, iden);
+    dlR = mulc<T>(rdL * du + dp, iden);
     SM = wl[1] + dlL;
     pts = ptL + rdL * dlL;
   }
@@ -1137,7 +1142,7 @@ __device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, cons
   const T bt = left ? btL : btR, v2 = u * u + v * v + vw * vw;
   const T hb = half<T>(left ? bbL : bbR), pt = left ? ptL : ptR;
   const T e = w[4] * gm1i + (half<T>(r) * v2 + hb);
-  const T mu = r * u;
+  const T mu = mulc<T>(r, u);
   const T vby = v * by + vw * bz;
 
   // reverse of the physical flux of the selected side, and the cotangents of
@@ -1152,16 +1157,16 @@ __device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, cons
     rd = left ? rdL : rdR;
     Sd = S - SM;
     iSd = trcp<T>(Sd);
-    rs = rd * iSd;
+    rs = mulc<T>(rd, iSd);
     const T D = rd * Sd - bn2;
     if (!abs_lt<T>(D, Eps<T>::hlld * pts)) {
       iD = trcp<T>(D);
-      z = dl * iD;
+      z = mulc<T>(dl, iD);
     }
-    t = bn * z;
-    rz = rd * z;
-    m1 = S * (r * (dl * iSd));
-    C = bn + S * rs * t;
+    t = mulc<T>(bn, z);
+    rz = mulc<T>(rd, z);
+    m1 = mulc<T>(S, mulc<T>(r, mulc<T>(dl, iSd)));
+    C = bn + mulc<T>(S, rs) * t;
     A = u + S * rz;
     rsq = trsqrt<T>(rs);
     const T cA = fabs(bn) * rsq;
@@ -1192,35 +1197,35 @@ __device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, cons
       const T rdo = left ? rdR : rdL, dlo = left ? dlR : dlL;
       const T Sdo = (left ? SR : SL) - SM;
       const T iSdo = trcp<T>(Sdo);
-      const T rso = rdo * iSdo;
+      const T rso = mulc<T>(rdo, iSdo);
       const T Do = rdo * Sdo - bn2;
       T iDo = T(0);
       if (!abs_lt<T>(Do, Eps<T>::hlld * pts)) iDo = trcp<T>(Do);
-      const T zo = dlo * iDo;
-      const T q = T(1) + rz, to = bn * zo, qo = T(1) + rdo * zo;
+      const T zo = mulc<T>(dlo, iDo);
+      const T q = T(1) + rz, to = mulc<T>(bn, zo), qo = T(1) + rdo * zo;
       const T vs = v - by * t, ws = vw - bz * t, bys = by * q, bzs = bz * q;
       const T vo = wo[2] - wo[5] * to, wwo = wo[3] - wo[6] * to;
       const T rsqo = trsqrt<T>(rso);
-      const T sq = rs * rsq, sqo = rso * rsqo;
+      const T sq = mulc<T>(rs, rsq), sqo = mulc<T>(rso, rsqo);
       const T inv = trcp<T>(sq + sqo);
       const T sg = (gt0<T>(bn) == left) ? T(1) : T(-1);
       const T dv = vo - vs, dw = wwo - ws;
       const T Dy = (times_sign<T>(wo[5] * qo - bys, sg) + sqo * dv) * inv;
       const T Dz = (times_sign<T>(wo[6] * qo - bzs, sg) + sqo * dw) * inv;
       const T gg = times_sign<T>(sq, sg);
-      const T ay = Ss * Dy, az = Ss * Dz;
+      const T ay = mulc<T>(Ss, Dy), az = mulc<T>(Ss, Dz);
       const T vd = vs + Dy, wd = ws + Dz;
       const T Py = bys + gg * vd, Pz = bzs + gg * wd;
       // reverse
       g_rs += gf[2] * ay + gf[3] * az;
-      const T g4g = gf[4] * gg;
+      const T g4g = mulc<T>(gf[4], gg);
       const T g_ay = gf[2] * rs + g4g * Py + gf[5] * gg, g_az = gf[3] * rs + g4g * Pz + gf[6] * gg;
-      const T gPy = g4g * ay, gPz = g4g * az;
+      const T gPy = mulc<T>(g4g, ay), gPz = mulc<T>(g4g, az);
       const T g_gg = gf[4] * (ay * Py + az * Pz) + gf[5] * ay + gf[6] * az + (gPy * vd + gPz * wd);
       T g_vs = gPy * gg, g_ws = gPz * gg;
       const T g_Dy = g_vs + g_ay * Ss, g_Dz = g_ws + g_az * Ss;
       const T g_Ss = g_ay * Dy + g_az * Dz;
-      const T ny = g_Dy * inv, nz = g_Dz * inv;
+      const T ny = mulc<T>(g_Dy, inv), nz = mulc<T>(g_Dz, inv);
       const T g_sum = -(ny * Dy + nz * Dz);
       const T hy = times_sign<T>(ny, sg), hz = times_sign<T>(nz, sg);
       const T g_bys = gPy - hy, g_bzs = gPz - hz;
@@ -1231,13 +1236,13 @@ __device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, cons
       T g_sq = g_sum + times_sign<T>(g_gg, sg);
       // Ss = S_M -+ |bn| / sq
       g_SM += g_Ss;
-      const T gr = g_Ss * rsq;
+      const T gr = mulc<T>(g_Ss, rsq);
       const T sb = gt0<T>(bn) == left ? T(-1) : T(1);
       g_bn += times_sign<T>(gr, sb);
       const T ga = gr * (fabs(bn) * rsq);
       g_sq = left ? T(g_sq + ga) : T(g_sq - ga);
       g_rs += half<T>(g_sq) * rsq;
-      const T g_rso = half<T>(g_sqo) * rsqo;
+      const T g_rso = mulc<T>(half<T>(g_sqo), rsqo);
       // star state of the selected side
       g_v += g_vs;
       g_vw += g_ws;
@@ -1255,59 +1260,60 @@ __device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, cons
       const T g_qo = g_byo * wo[5] + g_bzo * wo[6];
       g_bn += g_to * zo;
       const T g_zo = g_to * bn + g_qo * rdo;
-      g_dlo = g_zo * iDo;
-      const T g_Do = -(g_zo * zo * iDo);
+      g_dlo = mulc<T>(g_zo, iDo);
+      const T g_Do = -mulc<T>(g_dlo, zo);
       g_rdo = g_qo * zo + g_Do * Sdo + g_rso * iSdo;
       g_So = g_Do * rdo - g_rso * rso * iSdo;
       g_SM -= g_So;
       g_bn -= twice<T>(bn * g_Do);
     }
     // dE = S K iSd, K = (e + p* + u rd) dl - bn dvb
-    const T bbt = bt * t;
+    const T bbt = mulc<T>(bt, t);
     const T dvb = rz * (vby - bbt) + (bn * dl - bbt);
     const T H = e + (pt + rd * dl) + u * rd;
     const T K = H * dl - bn * dvb;
     const T gE = gf[4];
-    const T gES = gE * S;
+    const T gES = mulc<T>(gE, S);
     g_S += gE * (K * iSd);
     g_iSd += gES * K;
-    const T gK = gES * iSd;
+    const T gK = mulc<T>(gES, iSd);
     g_dl += gK * H;
-    const T gH = gK * dl;
+    const T gH = mulc<T>(gK, dl);
     g_e += gH;
     g_pt += gH;
     g_u += gH * rd;
     g_rd += gH * (u + dl);
     g_dl += gH * rd;
-    const T gdvb = -(gK * bn);
+    const T gdvb = -mulc<T>(gK, bn);
     g_bn += gdvb * dl - gK * dvb;
     g_dl += gdvb * bn;
     g_vby += gdvb * rz;
     g_rz += gdvb * (vby - bbt);
-    const T gbbt = -(gdvb * (T(1) + rz));
+    const T gbbt = -mulc<T>(gdvb, T(1) + rz);
     g_bt += gbbt * t;
     g_t += gbbt * bt;
     // A = u + S rz, C = bn + S rs t
     g_S += gA * rz;
     g_rz += gA * S;
-    const T gCS = gC * S;
+    const T gCS = mulc<T>(gC, S);
     g_S += gC * (rs * t);
     g_rs += gCS * t;
     g_t += gCS * rs;
     // m1 = S r dl iSd, entering f0 (gf0) and, times S, f1
     const T g_m1 = gf0 + gf[1] * S;
-    const T h = dl * iSd, gh = g_m1 * S;
+    const T h = mulc<T>(dl, iSd), gh = mulc<T>(g_m1, S);
     g_S += g_m1 * (r * h) + gf[1] * m1;
     g_r += gh * h;
-    const T ghr = gh * r;
+    const T ghr = mulc<T>(gh, r);
     g_dl += ghr * iSd;
     g_iSd += ghr * dl;
     // rz = rd z, t = bn z, z = dl / D, D = rd Sd - bn2, rs = rd iSd
     g_rd += g_rz * z;
     g_bn += g_t * z;
     const T g_z = g_rz * rd + g_t * bn;
-    g_dl += g_z * iD;
-    const T g_D = -(g_z * z * iD);
+    const T gzD = mulc<T>(g_z, iD);
+    g_dl += gzD;
+    const T g_D = -mulc<T>(gzD, z);
     g_rd += g_D * Sd + g_rs * iSd;
     g_iSd += g_rs * rd;
     const T g_Sd = g_D * rd - g_iSd * iSd * iSd;
@@ -1321,8 +1327,8 @@ __device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, cons
   g_bz += g_vby * vw;
   // e = p gm1i + r v^2 / 2 + bb / 2, pt = p + bb / 2, bb = bn2 + bt
   T g_p = g_e * gm1i + g_pt;
-  const T ger = g_e * r;
-  g_r += half<T>(g_e * v2);
+  const T ger = mulc<T>(g_e, r);
+  g_r += half<T>(mulc<T>(g_e, v2));
   g_u += ger * u;
   g_v += ger * v;
   g_vw += ger * vw;
@@ -1332,7 +1338,7 @@ __device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, cons
     // middle wave: dl_L = (rd_R du + dp) iden, dl_R = (rd_L du + dp) iden, S_M = u_L + dl_L
     T g_dlL = left ? g_dl : g_dlo, g_dlR = left ? g_dlo : g_dl;
     g_dlL += g_SM;
-    const T nL = g_dlL * iden, nR = g_dlR * iden;
+    const T nL = mulc<T>(g_dlL, iden), nR = mulc<T>(g_dlR, iden);
     const T g_den = -(nL * dlL + nR * dlR);
     const T du = wr[1] - wl[1];
     T g_rdL = left ? g_rd : g_rdo, g_rdR = left ? g_rdo : g_rd;
@@ -1340,7 +1346,7 @@ __device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, cons
     g_rdL += nR * du - g_den;
     const T g_du = nL * rdR + nR * rdL, g_dp = nL + nR;
     // rd = rho (S - u)
-    const T aL = g_rdL * wl[0], aR = g_rdR * wr[0];
+    const T aL = mulc<T>(g_rdL, wl[0]), aR = mulc<T>(g_rdR, wr[0]);
     const T g_uL = g_SM - g_du - aL, g_uR = g_du - aR;
     const T g_rL = g_rdL * (SL - wl[1]), g_rR = g_rdR * (SR - wr[1]);
     T g_SL = left ? g_S : g_So, g_SR = left ? g_So : g_S;
@@ -1362,19 +1368,19 @@ __device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, cons
     g_uo += (left == lo ? T(0) : g_SL) + (left == hi ? T(0) : g_SR);
     // cmax^2 = X / (2 rho), X = gamma P + bb + s, s = sqrt((gamma P - bb)^2 + 4 gamma P bt)
     if (gt0<T>(cmax)) {
-      const T g_c2 = half<T>(g_c) * trcp<T>(cmax);
-      const T g_hX = g_c2 * irc;  // of X / 2
+      const T g_c2 = mulc<T>(half<T>(g_c), trcp<T>(cmax));
+      const T g_hX = mulc<T>(g_c2, irc);  // of X / 2
       const T gg = half<T>(g_hX);
       const T gp = gamma * (lmax ? wl[4] : wr[4]), bbm = lmax ? bbL : bbR, btm = lmax ? btL : btR, sm = lmax ? sL : sR;
       T g_gp = gg, g_bbm = gg, g_btm = T(0);
       if (gt0<T>(sm)) {
-        const T is = gg * trcp<T>(sm);
+        const T is = mulc<T>(gg, trcp<T>(sm));
         const T dd = gp - bbm;
         g_gp += is * (dd + twice<T>(btm));
         g_bbm -= is * dd;
-        g_btm = twice<T>(is * gp);
+        g_btm = twice<T>(mulc<T>(is, gp));
       }
-      const T g_rm = -(g_hX * c2), g_pm = gamma * g_gp;
+      const T g_rm = -mulc<T>(g_hX, c2), g_pm = mulc<T>(gamma, g_gp);
       const bool own = lmax == left;
       g_r += own ? g_rm : T(0);
       g_ro += own ? T(0) : g_rm;

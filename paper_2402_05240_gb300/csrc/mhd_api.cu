@@ -91,7 +91,14 @@ void padded_dims(const mhd_config& c, int n[3], int lo[3]) {
 
 size_t red_blocks(long long N) { return (size_t)mhd::diag_blocks(N); }
 
-Layout layout_of(const mhd_config& c) {
+// three-axis launches for this grid (they need W_L and W_R of all axes at once)
+bool wants_fuse(const mhd_config& c) {
+  int np[3], lo[3];
+  padded_dims(c, np, lo);
+  return mhd::fuse_axes(np[0], np[1], np[2]);
+}
+
+Layout layout_of(const mhd_config& c, bool fuse) {
   int np[3], lo[3];
   padded_dims(c, np, lo);
   const size_t N = (size_t)np[0] * np[1] * np[2];
@@ -105,7 +112,7 @@ Layout layout_of(const mhd_config& c) {
   off += up(21 * N * ts);
   L.E = off;
   off += up(3 * N * ts);
-  const size_t faces = mhd::fuse_axes(np[0], np[1], np[2]) ? 21 : 7;
+  const size_t faces = fuse ? 21 : 7;
   L.WL = off;
   off += up(faces * N * ts);
   L.WR = off;
@@ -594,7 +601,7 @@ int mhd_workspace_bytes(const mhd_config* cfg, size_t* bytes) {
   int st = check_cfg(cfg);
   if (st != MHD_OK) return st;
   if (!bytes) return MHD_ERR_ARG;
-  *bytes = layout_of(*cfg).total;
+  *bytes = layout_of(*cfg, wants_fuse(*cfg)).total;
   return MHD_OK;
 }
 
@@ -637,15 +644,22 @@ int mhd_init(mhd_ctx** out, const mhd_config* cfg, void* stream) {
   }
   c->stream = static_cast<cudaStream_t>(stream);
   c->ts = cfg->precision == MHD_FP32_BULK ? 4 : 8;
-  c->fuse = mhd::fuse_axes(np[0], np[1], np[2]);
-  const Layout L = layout_of(*cfg);
-  c->ws_bytes = L.total;
+  c->fuse = wants_fuse(*cfg);
+  Layout L = layout_of(*cfg, c->fuse);
   cudaGetLastError();
-  if (cudaMalloc(&c->ws, L.total) != cudaSuccess) {
+  cudaError_t got = cudaMalloc(&c->ws, L.total);
+  if (got != cudaSuccess && c->fuse) {  // one launch per axis where the larger workspace does not fit
+    cudaGetLastError();
+    c->fuse = false;
+    L = layout_of(*cfg, false);
+    got = cudaMalloc(&c->ws, L.total);
+  }
+  if (got != cudaSuccess) {
     cudaGetLastError();
     delete c;
     return MHD_ERR_OOM;
   }
+  c->ws_bytes = L.total;
   char* b = static_cast<char*>(c->ws);
   c->W = b + L.W;
   c->F = b + L.F;

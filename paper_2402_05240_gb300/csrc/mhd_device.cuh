@@ -250,6 +250,22 @@ template <> __device__ __forceinline__ double ratio_le1<double>(double a, double
   return r;
 }
 
+// A product that no sum takes up, as a call on the integer pipes (double; any
+// operands) -- see Ops
+static __device__ __noinline__ double mul_call(double a, double b) {
+  bool bad = false;
+  double r = mul_try(a, b, bad);
+  if (__any_sync(__activemask(), bad)) {
+    if (bad) r = mul_other(a, b);
+  }
+  return r;
+}
+// (float pairs: the unnormalised product, which a sum may take as it stands)
+template <class T> __device__ __forceinline__ auto mulc(T a, T b) {
+  if constexpr (std::is_same<T, double>::value) return mul_call(a, b);
+  else return a * b;
+}
+
 // The operations of the reconstruction and the Riemann solver that have more
 // than one form.  Ops: complete functions.  TryOps<double>: the integer-pipe
 // functions alone; `bad` tells that an operand left their range, and the
@@ -258,17 +274,28 @@ template <> __device__ __forceinline__ double ratio_le1<double>(double a, double
 // products that no sum takes up (a multiply-add is one FP64 instruction
 // anyway): on the integer pipes a product costs about 38 issue slots against
 // the 64 of an FP64 instruction, and the FP64 pipe has the less idle time.
-// Measured at 256^3, FP64: Riemann kernels (30 products of 120 operations) 10.9
-// -> 9.1 ms, PLMC reconstruction 23.9 -> 20.2 ms, PPMC 41.4 -> 33.2 ms (31
-// products of the eigensystem and 8 of each projection, as calls: CallOps).
+// The product is a call, operands and result in registers: inlined, its copies
+// spill registers and outgrow the instruction cache (PPMC with the projections'
+// products 45.8 ms inlined, 33.2 ms as calls; Riemann kernels with 38 products
+// 10.2 and 8.7 ms).  Measured at 256^3, FP64: Riemann kernels 10.9 -> 8.7 ms, PLMC
+// reconstruction 23.9 -> 18.6 ms, PPMC 41.4 -> 32.6 ms.
 template <class T> struct Ops {
   static constexpr bool bad = false;
   __device__ __forceinline__ T rcp(T x) { return trcp<T>(x); }
   __device__ __forceinline__ T sqrt(T x) { return tsqrt<T>(x); }
   __device__ __forceinline__ T rsqrt(T x) { return trsqrt<T>(x); }
   __device__ __forceinline__ T quad(T x) { return mhd::quad<T>(x); }
-  __device__ __forceinline__ T mul(T a, T b) { return a * b; }
+  __device__ __forceinline__ auto mul(T a, T b) { return mulc<T>(a, b); }
 };
+struct TryValue {
+  double v;
+  int bad;
+};
+static __device__ __noinline__ TryValue mul_try_call(double a, double b) {
+  bool bad = false;
+  const double v = mul_try(a, b, bad);
+  return TryValue{v, bad};
+}
 template <class T> struct TryOps : Ops<T> {};
 template <> struct TryOps<double> {
   bool bad = false;
@@ -280,24 +307,6 @@ template <> struct TryOps<double> {
     bad |= (b != 0) & ((unsigned long long)(b - (1LL << 52)) >= (0x7fdULL << 52) - (1ULL << 52));
     return __longlong_as_double(b ? b + (2LL << 52) : b);
   }
-  __device__ __forceinline__ double mul(double a, double b) { return mul_try(a, b, bad); }
-};
-
-// TryOps with the product as a call, for the reconstruction: inlined, its
-// products spill registers and outgrow the instruction cache, so only those of
-// the eigensystem paid; as a call (operands and result in registers) those of
-// the projections do too.
-struct TryValue {
-  double v;
-  int bad;
-};
-static __device__ __noinline__ TryValue mul_try_call(double a, double b) {
-  bool bad = false;
-  const double v = mul_try(a, b, bad);
-  return TryValue{v, bad};
-}
-template <class T> struct CallOps : TryOps<T> {};
-template <> struct CallOps<double> : TryOps<double> {
   __device__ __forceinline__ double mul(double a, double b) {
     const TryValue r = mul_try_call(a, b);
     bad |= r.bad != 0;
@@ -491,7 +500,7 @@ __device__ __forceinline__ void hlld_jump(T gamma, T gm1i, const T* wl, const T*
 template <class T, class O>
 __device__ __forceinline__ void hlld_diff(O& o, T gamma, T gm1i, const T* wl, const T* wr, T bn, T* f) {
   const T bn2 = o.mul(bn, bn);
-  const T btL = wl[5] * wl[5] + wl[6] * wl[6], btR = wr[5] * wr[5] + wr[6] * wr[6];
+  const T btL = o.mul(wl[5], wl[5]) + wl[6] * wl[6], btR = o.mul(wr[5], wr[5]) + wr[6] * wr[6];
   const T bbL = bn2 + btL, bbR = bn2 + btR;
   const T ptL = wl[4] + half<T>(bbL), ptR = wr[4] + half<T>(bbR);
   // 2 rho c_f^2 = gamma P + B^2 + sqrt((gamma P - B^2)^2 + 4 gamma P B_t^2):
@@ -524,9 +533,9 @@ __device__ __forceinline__ void hlld_diff(O& o, T gamma, T gm1i, const T* wl, co
   const T* w = left ? wl : wr;
   const T r = w[0], u = w[1], v = w[2], vw = w[3], by = w[5], bz = w[6];
   const T pt = left ? ptL : ptR, bt = left ? btL : btR;
-  const T e = w[4] * gm1i + (half<T>(r) * (u * u + v * v + vw * vw) + half<T>(left ? bbL : bbR));
+  const T e = w[4] * gm1i + (half<T>(r) * (o.mul(u, u) + v * v + vw * vw) + half<T>(left ? bbL : bbR));
   const T mu = o.mul(r, u);
-  const T vby = v * by + vw * bz;
+  const T vby = o.mul(v, by) + vw * bz;
   // the increments S (U* - U) of the star region: zero for a supersonic face
   T m1 = T(0), sm1 = T(0), C = bn, A = u, dE = T(0);
   T rs = T(0), z = T(0), rd = T(0), Ss = T(0);
@@ -558,11 +567,11 @@ __device__ __forceinline__ void hlld_diff(O& o, T gamma, T gm1i, const T* wl, co
   const T f0 = mu + m1;
   f[0] = f0;
   f[1] = mu * u + (pt - bn2) + sm1;
-  f[2] = f0 * v - by * C;
-  f[3] = f0 * vw - bz * C;
-  f[4] = (e + pt) * u - bn * (u * bn + vby) + dE;
-  f[5] = by * A - bn * v;
-  f[6] = bz * A - bn * vw;
+  f[2] = o.mul(f0, v) - by * C;
+  f[3] = o.mul(f0, vw) - bz * C;
+  f[4] = o.mul(e + pt, u) - bn * (u * bn + vby) + dE;
+  f[5] = o.mul(by, A) - bn * v;
+  f[6] = o.mul(bz, A) - bn * vw;
   if (inner) {
     // the increments Ss (U** - U*) of the double-star region: with the star
     // states of both sides, Delta = v** - v* = (sgn(B_n) (B*_R - B*_L) +-
@@ -698,28 +707,45 @@ template <class T> __device__ __forceinline__ void eig_build(T gamma, const T* w
 
 // characteristic amplitudes q = L dw
 //
-// Double and float pairs take the products of the eigensystem's fields as
-// coefficients (the compiler forms them once per cell for all projections of
-// a reconstruction): 23 operations per projection against 35 in the form
+// Double and float pairs take products of the eigensystem's fields, formed
+// once for all projections of a cell (EigCoef), as coefficients: 23 operations per projection against 35 in the form
 // below, which float keeps (its rounding fixes the FP32-bulk mode's results).
 // With the shorter limiter below: FP64 PLMC 256^3 61.8 -> 56.1 ms per step,
 // double-float PPMC 512^3 193 -> 182 ms.
-template <class T, class O> __device__ __forceinline__ void eig_left(O& o, const Eig<T>& E, const T* dw, T* q) {
+// EigCoef: the fast and slow amplitudes of dP (fp, sp), of dB along beta (fb,
+// sb) and of du (fu, su; of dv along beta su, fu), the Alfven ones of dv (h)
+// and dB (z).
+template <class T> struct EigCoef {
+  T fp, sp, fb, sb, fu, su, h1, h2, z1, z2;
+};
+template <class T, class O> __device__ __forceinline__ EigCoef<T> eig_coef(O& o, const Eig<T>& E) {
+  EigCoef<T> C;
   if constexpr (sizeof(T) != 4) {
     const T n = half<T>(E.ia2);
     const T naf = o.mul(n, E.af), nas = o.mul(n, E.as), ai = o.mul(E.a, E.isr);
-    const T fp = o.mul(naf, E.ir), sp = o.mul(nas, E.ir);    // fast, slow amplitude of dP
-    const T fb = o.mul(nas, ai), sb = o.mul(naf, ai);        // of dB along beta
-    const T fu = o.mul(naf, E.cf), su = o.mul(nas, E.cs);    // of du (and of dv along beta: su, fu)
-    const T h1 = half<T>(E.b1), h2 = half<T>(E.b2);
     const T z = times_sign<T>(E.isr, E.sg);
-    const T z1 = o.mul(h1, z), z2 = o.mul(h2, z);
+    C.fp = o.mul(naf, E.ir);
+    C.sp = o.mul(nas, E.ir);
+    C.fb = o.mul(nas, ai);
+    C.sb = o.mul(naf, ai);
+    C.fu = o.mul(naf, E.cf);
+    C.su = o.mul(nas, E.cs);
+    C.h1 = half<T>(E.b1);
+    C.h2 = half<T>(E.b2);
+    C.z1 = o.mul(C.h1, z);
+    C.z2 = o.mul(C.h2, z);
+  }
+  return C;
+}
+template <class T, class O>
+__device__ __forceinline__ void eig_left(O& o, const Eig<T>& E, const EigCoef<T>& C, const T* dw, T* q) {
+  if constexpr (sizeof(T) != 4) {
     const T bv = times_sign<T>(o.mul(E.b1, dw[2]) + E.b2 * dw[3], E.sg);
     const T bb = o.mul(E.b1, dw[5]) + E.b2 * dw[6];
-    const T Xf = o.mul(fp, dw[4]) + fb * bb, Yf = o.mul(su, bv) - fu * dw[1];
-    const T Xs = o.mul(sp, dw[4]) - sb * bb, Ys = o.mul(su, dw[1]) + fu * bv;
-    const T Z = o.mul(h1, dw[3]) - h2 * dw[2];
-    const T Zb = o.mul(z1, dw[6]) - z2 * dw[5];
+    const T Xf = o.mul(C.fp, dw[4]) + C.fb * bb, Yf = o.mul(C.su, bv) - C.fu * dw[1];
+    const T Xs = o.mul(C.sp, dw[4]) - C.sb * bb, Ys = o.mul(C.su, dw[1]) + C.fu * bv;
+    const T Z = o.mul(C.h1, dw[3]) - C.h2 * dw[2];
+    const T Zb = o.mul(C.z1, dw[6]) - C.z2 * dw[5];
     q[0] = Xf + Yf;
     q[1] = Z + Zb;
     q[2] = Xs - Ys;
@@ -749,9 +775,9 @@ template <class T, class O> __device__ __forceinline__ void eig_left(O& o, const
   q[6] = n * (Xf - Yf);
 }
 
-template <class T> __device__ __forceinline__ void eig_left(const Eig<T>& E, const T* dw, T* q) {
+template <class T> __device__ __forceinline__ void eig_left(const Eig<T>& E, const EigCoef<T>& C, const T* dw, T* q) {
   Ops<T> o;
-  eig_left<T>(o, E, dw, q);
+  eig_left<T>(o, E, C, dw, q);
 }
 
 // primitive increments dw = R q
@@ -863,9 +889,10 @@ __device__ __forceinline__ void plmc(O& o, T gamma, const T* wm, const T* w0, co
   Eig<T> E;
   eig_build<T>(o, gamma, w0, bn, E);
   T aL[7], aR[7], aC[7], aG[7], am[7], dW[7];
-  eig_left<T>(o, E, dL, aL);
-  eig_left<T>(o, E, dR, aR);
-  eig_left<T>(o, E, dG, aG);
+  const EigCoef<T> C = eig_coef<T>(o, E);
+  eig_left<T>(o, E, C, dL, aL);
+  eig_left<T>(o, E, C, dR, aR);
+  eig_left<T>(o, E, C, dG, aG);
   // the centred difference (W_{i+1} - W_{i-1})/2 projected: L is linear, so
   // its amplitudes are the mean of the left and right ones
 #pragma unroll
@@ -1050,6 +1077,7 @@ template <class T, class O>
 __device__ __forceinline__ void ppmc(O& o, T gamma, const T (*w)[7], T bn, T* wl, T* wr) {
   Eig<T> E;
   eig_build<T>(o, gamma, w[2], bn, E);
+  const EigCoef<T> C = eig_coef<T>(o, E);
   T qs[5][7];
 #pragma unroll
   for (int m = 0; m < 5; ++m) {
@@ -1061,7 +1089,7 @@ __device__ __forceinline__ void ppmc(O& o, T gamma, const T (*w)[7], T bn, T* wl
     T d[7];
 #pragma unroll
     for (int c = 0; c < 7; ++c) d[c] = w[m][c] - w[2][c];
-    eig_left<T>(o, E, d, qs[m]);
+    eig_left<T>(o, E, C, d, qs[m]);
   }
   T dm[7], dp[7];
 #pragma unroll

@@ -181,6 +181,7 @@ __device__ __forceinline__ double mul_try(double a, double b, bool& bad) {
 static __device__ __noinline__ double rcp_other(double x) { return __drcp_rn(x); }
 static __device__ __noinline__ double sqrt_other(double x) { return __dsqrt_rn(x); }
 static __device__ __noinline__ double rsqrt_other(double x) { return rsqrt(x); }
+static __device__ __noinline__ double mul_other(double a, double b) { return a * b; }
 __device__ __forceinline__ double rcp_int(double x) {
   bool bad = false;
   double r = rcp_try(x, bad);

@@ -517,7 +517,7 @@ __device__ __noinline__ void recon_cell_again(const Grid& g, const Fields<const 
 }
 template <class T, int RECON, int A>
 __device__ __forceinline__ void recon_cell(const Grid& g, const Fields<const T, 8>& W, const Cell& p, T* wl, T* wr) {
-  CallOps<T> o;
+  TryOps<T> o;
   recon_cell_with<T, RECON, A>(o, g, W, p, wl, wr);
   if constexpr (std::is_same<T, double>::value && (RECON == 1 || RECON == 2)) {
     if (__any_sync(__activemask(), o.bad)) {
