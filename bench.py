@@ -80,43 +80,43 @@ ISSUE_PEAK_GWARPINST = 4 * 152 * 2.07
 # bytes read + written).  They hold for the kernels as profiled; a kernel
 # changed since has no entry.  The PCM predictor, edge fields, updates and
 # primitives do not depend on the reconstruction; PLMC has no reconstruction
-# entry (its kernel changed after its capture).
+# entry (its kernel was not captured).
 _STAGES = {
     "fp64": {
-        "prim": (45.7, 65.1, 1020.3 / 32, 145.0),
-        "flux_pcm": (232.6, 350.8, 1416.9 / 32, 114.2),
-        "emf": (48.0, 51.0, 698.0 / 32, 118.3),
-        "update_half": (92.0, 133.0, 646.0 / 32, 315.6),
-        "flux_hlld": (232.1, 349.9, 1422.6 / 32, 171.9),
-        "update_full": (45.0, 66.0, 352.0 / 32, 268.3),
+        "prim": (21.0, 29.0, 893.1 / 32, 144.4),
+        "flux_pcm": (81.3, 117.4, 4006.7 / 32, 114.2),
+        "emf": (33.0, 33.0, 631.0 / 32, 118.3),
+        "update_half": (81.0, 116.0, 696.0 / 32, 315.6),
+        "flux_hlld": (81.2, 117.2, 4015.1 / 32, 172.0),
+        "update_full": (45.0, 66.0, 356.0 / 32, 268.5),
     },
     "fp32_bulk": {
-        "prim": (18.0, 29.0, 719.0 / 32, 102.5),
-        "flux_pcm": (0.0, 0.0, 493.3 / 32, 58.8),
-        "emf": (0.0, 0.0, 224.0 / 32, 58.0),
-        "update_half": (29.0, 46.0, 1103.0 / 32, 188.5),
-        "flux_hlld": (0.0, 0.0, 524.2 / 32, 84.3),
-        "update_full": (16.0, 19.0, 1040.8 / 32, 194.4),
+        "prim": (12.0, 18.0, 779.0 / 32, 102.5),
+        "flux_pcm": (0.0, 0.0, 495.3 / 32, 58.8),
+        "emf": (0.0, 0.0, 223.0 / 32, 58.1),
+        "update_half": (23.0, 35.0, 1145.0 / 32, 188.5),
+        "flux_hlld": (0.0, 0.0, 526.2 / 32, 84.3),
+        "update_full": (16.0, 19.0, 1049.1 / 32, 194.3),
     },
     "fp64_df": {
-        "prim": (37.0, 53.0, 1517.3 / 32, 144.2),
-        "flux_pcm": (0.0, 0.0, 2876.8 / 32, 114.2),
-        "emf": (0.0, 0.0, 801.9 / 32, 118.2),
-        "update_half": (45.0, 62.0, 2051.0 / 32, 315.5),
-        "flux_hlld": (0.0, 0.0, 2816.5 / 32, 172.0),
-        "update_full": (16.0, 19.0, 1145.0 / 32, 268.1),
+        "prim": (15.0, 20.0, 952.5 / 32, 144.4),
+        "flux_pcm": (0.0, 0.0, 1987.3 / 32, 114.0),
+        "emf": (0.0, 0.0, 732.4 / 32, 118.2),
+        "update_half": (37.0, 48.0, 2019.0 / 32, 315.5),
+        "flux_hlld": (0.0, 0.0, 1970.7 / 32, 171.8),
+        "update_full": (16.0, 19.0, 1096.0 / 32, 268.1),
     },
 }
 # FP64-pipe busy fraction of the FP64 kernels from the same captures
 # (sm__pipe_fp64_cycles_active, % of peak sustained active): the pipe's
 # occupancy by every FP64 instruction issued -- arithmetic, compares, and the
 # lanes a divergent branch leaves idle -- beside the algorithmic count above
-FP64_PIPE_BUSY = {"prim": 0.858, "flux_pcm": 0.892, "emf": 0.838, "update_half": 0.870, "recon": 0.852,
-                  "flux_hlld": 0.892, "update_full": 0.879}
+FP64_PIPE_BUSY = {"prim": 0.845, "flux_pcm": 0.802, "emf": 0.837, "update_half": 0.874, "recon": 0.842,
+                  "flux_hlld": 0.793, "update_full": 0.882}
 _RECON_PPMC = {
-    "fp64": (420.2, 529.6, 3675.0 / 32, 169.6),
-    "fp32_bulk": (0.0, 0.0, 1260.9 / 32, 80.9),
-    "fp64_df": (0.0, 0.0, 7048.3 / 32, 169.4),
+    "fp64": (261.5, 348.3, 9340.4 / 32, 178.8),
+    "fp32_bulk": (0.0, 0.0, 1262.9 / 32, 80.9),
+    "fp64_df": (0.0, 0.0, 5313.3 / 32, 169.3),
 }
 COUNTERS = {
     "plmc": {prec: dict(tab) for prec, tab in _STAGES.items()},
