@@ -111,7 +111,9 @@ int mhd_workspace_bytes(const mhd_config* cfg, size_t* bytes);
 /* Library infrastructure, not in the paper.  Creates a context for cfg on
  * the current CUDA device; stream is a cudaStream_t (NULL = default stream)
  * that every later call on the context uses.  Allocates and zeroes the
- * workspace (mhd_workspace_bytes) and synchronises the stream.  *out
+ * workspace (mhd_workspace_bytes; grids of up to 128^3 cells fall back to a
+ * smaller one, 28 words per cell less, where that cannot be allocated: one
+ * launch per axis) and synchronises the stream.  *out
  * receives the context (owned by the caller, freed by mhd_destroy), or NULL
  * on error.  Errors: MHD_ERR_ARG (out or cfg NULL, cfg invalid),
  * MHD_ERR_OOM (host or device allocation failed), MHD_ERR_CUDA. */
