@@ -56,13 +56,13 @@ __global__ void __launch_bounds__(BX* BY) k_adj_floors(Grid g, const double* __r
   const StepScalars S = step_scalars_of(g, dt);
   double u5[5];
   constexpr bool X = Exact<T>::full;  // the arithmetic of k_update_full
-  hydro_update<T, X, true, false>(Uf, Ff, S, p, u5);
-  const double bx = face_update<T, X, true, 0>(g, Uf, Ef, S.dt, c, p.m[1], p.m[2]);
-  const double by = face_update<T, X, true, 1>(g, Uf, Ef, S.dt, c, p.m[2], p.m[0]);
-  const double bz = face_update<T, X, true, 2>(g, Uf, Ef, S.dt, c, p.m[0], p.m[1]);
-  const double bxm = face_update<T, X, true, 0>(g, Uf, Ef, S.dt, c + p.m[0], p.m[1], p.m[2]);
-  const double bym = face_update<T, X, true, 1>(g, Uf, Ef, S.dt, c + p.m[1], p.m[2], p.m[0]);
-  const double bzm = face_update<T, X, true, 2>(g, Uf, Ef, S.dt, c + p.m[2], p.m[0], p.m[1]);
+  hydro_update<T, X, false>(Uf, Ff, S, p, u5);
+  const double bx = face_update<T, X, 0>(g, Uf, Ef, S.dt, c, p.m[1], p.m[2]);
+  const double by = face_update<T, X, 1>(g, Uf, Ef, S.dt, c, p.m[2], p.m[0]);
+  const double bz = face_update<T, X, 2>(g, Uf, Ef, S.dt, c, p.m[0], p.m[1]);
+  const double bxm = face_update<T, X, 0>(g, Uf, Ef, S.dt, c + p.m[0], p.m[1], p.m[2]);
+  const double bym = face_update<T, X, 1>(g, Uf, Ef, S.dt, c + p.m[1], p.m[2], p.m[0]);
+  const double bzm = face_update<T, X, 2>(g, Uf, Ef, S.dt, c + p.m[2], p.m[0], p.m[1]);
   const double b[3] = {0.5 * (bxm + bx), 0.5 * (bym + by), 0.5 * (bzm + bz)};
   double g5[5];
 #pragma unroll
@@ -677,13 +677,13 @@ __global__ void __launch_bounds__(BX* BY) k_fwd_half_keep(Grid g, const double* 
   const double h = S.h_half;
   constexpr bool X = sizeof(T) == 8 && Exact<T>::full;  // the arithmetic of k_update_half
   double u5[5];
-  hydro_update<T, X, true, true>(Uf, Ff, S, p, u5);
-  const double bx = face_update<T, X, true, 0>(g, Uf, Ef, h, c, p.m[1], p.m[2]);
-  const double by = face_update<T, X, true, 1>(g, Uf, Ef, h, c, p.m[2], p.m[0]);
-  const double bz = face_update<T, X, true, 2>(g, Uf, Ef, h, c, p.m[0], p.m[1]);
-  const double bxm = face_update<T, X, true, 0>(g, Uf, Ef, h, c + p.m[0], p.m[1], p.m[2]);
-  const double bym = face_update<T, X, true, 1>(g, Uf, Ef, h, c + p.m[1], p.m[2], p.m[0]);
-  const double bzm = face_update<T, X, true, 2>(g, Uf, Ef, h, c + p.m[2], p.m[0], p.m[1]);
+  hydro_update<T, X, true>(Uf, Ff, S, p, u5);
+  const double bx = face_update<T, X, 0>(g, Uf, Ef, h, c, p.m[1], p.m[2]);
+  const double by = face_update<T, X, 1>(g, Uf, Ef, h, c, p.m[2], p.m[0]);
+  const double bz = face_update<T, X, 2>(g, Uf, Ef, h, c, p.m[0], p.m[1]);
+  const double bxm = face_update<T, X, 0>(g, Uf, Ef, h, c + p.m[0], p.m[1], p.m[2]);
+  const double bym = face_update<T, X, 1>(g, Uf, Ef, h, c + p.m[1], p.m[2], p.m[0]);
+  const double bzm = face_update<T, X, 2>(g, Uf, Ef, h, c + p.m[2], p.m[0], p.m[1]);
   Bh[c] = from_d<T>(bx);
   Bh[N + c] = from_d<T>(by);
   Bh[2 * N + c] = from_d<T>(bz);
