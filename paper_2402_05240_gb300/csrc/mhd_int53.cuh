@@ -112,17 +112,26 @@ MHD_INT_HD uint64_t mul_sig(uint64_t a, uint64_t b, int& big) {
   return (hi + (((1ull << sh) >> 1) - 1 + ((hi >> sh) & 1))) >> sh;
 }
 
-#if defined(__CUDACC__)
+// (MHD_HOST_CHECK: compiled for the host against stand-ins of the builtins)
+#if defined(__CUDACC__) || defined(MHD_HOST_CHECK)
 
 __device__ __forceinline__ float rcp_seed(float x) {
+#if defined(MHD_HOST_CHECK)
+  return 1.0f / x;
+#else
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
+#endif
 }
 __device__ __forceinline__ float rsqrt_seed(float x) {
+#if defined(MHD_HOST_CHECK)
+  return 1.0f / std::sqrt(x);
+#else
   float r;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
+#endif
 }
 
 __device__ __forceinline__ uint64_t sig53(int hi, int lo) {
@@ -207,6 +216,6 @@ __device__ __forceinline__ double sqrt_int(double x) {
   return r;
 }
 
-#endif  // __CUDACC__
+#endif  // __CUDACC__ || MHD_HOST_CHECK
 
 }  // namespace mhd
