@@ -867,6 +867,11 @@ template <class T, class O> __device__ __forceinline__ void van_leer7(O& o, cons
       const T pr = dL[q] * dR[q];
       const T g = twice<T>(pr) * o.rcp(act ? dL[q] + dR[q] : 1.0);
       dG[q] = (act && !is0<T>(pr)) ? g : T(0);
+    } else if constexpr (std::is_same<T, df>::value) {
+      // the sign from the product's leading float: pos_prod<df> holds for a
+      // product that underflows, too, where 1/s may leave the float range
+      const dfx pr = dL[q] * dR[q];
+      dG[q] = pr.hi > 0.0f ? T(T(2) * pr * o.rcp(dL[q] + dR[q])) : T(0);
     } else {
       dG[q] = pos_prod<T>(dL[q], dR[q]) ? T(2) * (dL[q] * dR[q]) * o.rcp(dL[q] + dR[q]) : T(0);
     }

@@ -86,3 +86,61 @@ int main() {
 
 def test_integer_pipe_functions(tmp_path):
     assert compile_and_run(tmp_path, INT_PIPE) == ["0", "0", "0"]
+
+
+TINY_DIFFERENCES = r"""
+// A cell with slopes of order one in density, normal velocity and pressure and
+// differences of size d in its transverse components, which are of order 1e-37
+// (a float pair made from a double below 2^-126 is zero; a difference of two
+// may be any subnormal).
+template <class T> static void cells(double d, T (*w)[7]) {
+  const double x = d == 0.0 ? 0.0 : 1e-37 + 4 * d;
+  const double base[7] = {1.0, 0.3, x, x, 0.8, x, x}, slope[7] = {0.2, -0.1, d, 1.5 * d, 0.15, 2.0 * d, -d};
+  for (int m = 0; m < 3; ++m)
+    for (int q = 0; q < 7; ++q) w[m][q] = T(base[q] + slope[q] * (m - 1) * (q < 2 || q == 4 ? 1.0 + 0.3 * (m - 1) : 1.0));
+}
+int main() {
+  typedef TYPE T;
+  long bad = 0;
+  for (double d : {1e-45, 1e-42, 5e-40, 1e-39, 2.5e-39, 3.5e-39, 1e-38, 1e-37, 1e-30, 1e-24, 1e-19}) {
+    T a[7], b[7], g[7];
+    for (int q = 0; q < 7; ++q) {
+      a[q] = T((float)(q & 1 ? d : -d));
+      b[q] = T((float)(q & 1 ? 0.5 * d : -0.5 * d));
+    }
+    van_leer7<T>(a, b, g);  // the harmonic mean 2 d / 3, or 0 where a product underflows
+    for (int q = 0; q < 7; ++q) {
+      const double x = fabs(to_d<T>(g[q]));
+      bad += !(x <= 1.01 * d + 1e-45);
+    }
+    T w[3][7], z[3][7], wl[7], wr[7], zl[7], zr[7];
+    cells<T>(d, w);
+    cells<T>(0.0, z);
+    Ops<T> o;
+    plmc<T>(o, T(5.0 / 3.0), w[0], w[1], w[2], T(0.4), wl, wr);
+    plmc<T>(o, T(5.0 / 3.0), z[0], z[1], z[2], T(0.4), zl, zr);
+    // differences of size d change the states by some d
+    for (int q = 0; q < 7; ++q) {
+      bad += !(fabs(to_d<T>(wl[q]) - to_d<T>(zl[q])) <= 1e-12 + 100 * d);
+      bad += !(fabs(to_d<T>(wr[q]) - to_d<T>(zr[q])) <= 1e-12 + 100 * d);
+    }
+    T gl[7], gr[7], gm[7], g0[7], gp[7], gbn = T(0);
+    for (int q = 0; q < 7; ++q) {
+      gl[q] = T(1.0 - 0.1 * q);
+      gr[q] = T(0.5 + 0.2 * q);
+      gm[q] = g0[q] = gp[q] = T(0);
+    }
+    plmc_vjp<T>(T(5.0 / 3.0), T(1e-20), T(1e-20), w[0], w[1], w[2], T(0.4), gl, gr, gm, g0, gp, gbn);
+    bad += !std::isfinite(to_d<T>(gbn));
+    for (int q = 0; q < 7; ++q)
+      bad += !std::isfinite(to_d<T>(gm[q])) + !std::isfinite(to_d<T>(g0[q])) + !std::isfinite(to_d<T>(gp[q]));
+  }
+  printf("%ld\n", bad);
+}
+"""
+
+
+@pytest.mark.parametrize("typ", ["df", "double", "float"])
+def test_plmc_with_tiny_differences(tmp_path, typ):
+    """Differences whose product underflows leave van Leer's mean at zero."""
+    assert compile_and_run(tmp_path, TINY_DIFFERENCES.replace("TYPE", typ)) == ["0"]
