@@ -1793,18 +1793,22 @@ __device__ void hlld_vjp(T gamma, const T* wl, const T* wr, T bn, const T* gf, T
 }
 
 // ------------------------------------------------- primitive recovery VJP --
-// W = (rho', v, P', B_cc) from (rho, m, E, B_cc) as in prim_core; gW[8]
-// cotangents; returns g of (rho, m0, m1, m2, E) in g5 and adds to gb[3].
-__device__ __forceinline__ void prim_vjp(const Grid& g, double r, double m0, double m1, double m2, double e,
+// W = (rho', v, P', B_cc) from (rho, m, E, B_cc) as in prim_core; pfl: the
+// forward holds P' at the floor (at_p_floor); gW[8] cotangents; returns g of
+// (rho, m0, m1, m2, E) in g5 and adds to gb[3].
+//
+// The decision is read off the pressure that the forward stored, not formed
+// again: where the kinetic and magnetic energy exceed the floor by 1 / eps, as in
+// every cell that a floor has just reset, it is the sign of a rounding error.
+template <class T> __device__ __forceinline__ bool at_p_floor(const Grid& g, T p) {
+  return !(p > from_d<T>(g.p_floor));
+}
+__device__ __forceinline__ void prim_vjp(const Grid& g, double r, double m0, double m1, double m2, bool pfl,
                                          const double* b, const double* gW, double* g5, double* gb) {
   const bool rfl = !(r >= g.rho_floor);  // fmax(r, floor) takes the floor
   const double rho = fmax(r, g.rho_floor);
   const double ir = trcp<double>(rho);  // (the correctly rounded 1/rho)
   const double v0 = m0 * ir, v1 = m1 * ir, v2 = m2 * ir;
-  const double ke = 0.5 * (m0 * v0 + m1 * v1 + m2 * v2);
-  const double me = 0.5 * (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
-  const double p = (g.gamma - 1.0) * (e - ke - me);
-  const bool pfl = !(p >= g.p_floor);
   const double gP = pfl ? 0.0 : gW[4];
   double grho = gW[0];
   double gv0 = gW[1], gv1 = gW[2], gv2 = gW[3];
@@ -1829,17 +1833,13 @@ __device__ __forceinline__ void prim_vjp(const Grid& g, double r, double m0, dou
   g5[4] = ge;
 }
 
-// The same reverse for the FP32-bulk mode: the floor decisions from the
-// double pressure recovery as the FP32-bulk forward forms it
-// (P = (gamma - 1)(E - (|m|^2 / rho' + |B_cc|^2) / 2)), the derivative
-// arithmetic in float; gb[3] is written, not accumulated.
-__device__ __forceinline__ void prim_vjp_f32(const Grid& g, double r, double m0, double m1, double m2, double e,
+// The same reverse for the FP32-bulk mode, the derivative arithmetic in float;
+// gb[3] is written, not accumulated.
+__device__ __forceinline__ void prim_vjp_f32(const Grid& g, double r, double m0, double m1, double m2, bool pfl,
                                              const double* b, const float* gW, float* g5, float* gb) {
   const bool rfl = !(r >= g.rho_floor);
   const double rho = fmax(r, g.rho_floor);
   const double ir = trcp<double>(rho);
-  const double kem = 0.5 * ((m0 * m0 + m1 * m1 + m2 * m2) * ir + (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]));
-  const bool pfl = !(g.gm1 * (e - kem) >= g.p_floor);
   const float irf = d2f_bits(ir), gm1 = d2f_bits(g.gm1);
   const float m[3] = {d2f_bits(m0), d2f_bits(m1), d2f_bits(m2)};
   const float bf[3] = {d2f_bits(b[0]), d2f_bits(b[1]), d2f_bits(b[2])};

@@ -71,22 +71,20 @@ __global__ void __launch_bounds__(BX* BY) k_adj_floors(Grid g, const double* __r
   const bool rfl = u5[0] < g.rho_floor;
   const double r = rfl ? g.rho_floor : u5[0];
   const double ir = trcp<double>(r);
-  // kinetic + magnetic energy and the pressure-floor test with the forward's
-  // arithmetic (k_prim; its FP32-bulk form in p_recover_f32)
-  double ke, me;
-  bool pfl;
+  // the pressure-floor test with the forward's functions (k_prim)
+  double ke, pe;
   if constexpr (std::is_same<T, float>::value) {
     ke = 0.5 * ((u5[1] * u5[1] + u5[2] * u5[2] + u5[3] * u5[3]) * ir);
-    me = 0.5 * (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
     const double bs[3] = {bxm + bx, bym + by, bzm + bz};
-    double t2, pe;
+    double t2;
     p_recover_f32(ir, u5[1], u5[2], u5[3], u5[4], bs, t2, pe);
-    pfl = lt_pos<double>(g.gm1 * pe, g.p_floor);
   } else {
-    ke = 0.5 * (u5[1] * (u5[1] * ir) + u5[2] * (u5[2] * ir) + u5[3] * (u5[3] * ir));
-    me = 0.5 * (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
-    pfl = g.gm1 * (u5[4] - ke - me) < g.p_floor;
+    const double v[3] = {u5[1] * ir, u5[2] * ir, u5[3] * ir};
+    double mv, bb;
+    p_recover(u5 + 1, v, u5[4], b, mv, bb, pe);
+    ke = 0.5 * mv;
   }
+  const bool pfl = lt_pos<double>(g.gm1 * pe, g.p_floor);
   if (pfl) {  // E = p_floor/(gamma-1) + |m|^2/(2 r) + |B_cc|^2/2
     const double gE = g5[4];
     g5[4] = 0.0;
@@ -598,25 +596,28 @@ __global__ void __launch_bounds__(BX* BY) k_adj_recon_gather(Grid g, const T* __
 
 // ------------------------------------------------ R5 / R10: primitives --
 // W = prim(hydro, B_cc): cotangent of the hydro fields (g5 out) and of B_cc
-// (gBcc out).  HALF: hydro from the stored half state; else from U^n.
+// (gBcc out).  HALF: hydro from the stored half state; else from U^n.  W: the
+// forward's primitives of the same state.
 template <class T, bool HALF>
 __global__ void __launch_bounds__(BX* BY) k_adj_prim(Grid g, const double* __restrict__ U, const double* __restrict__ Uh,
-                                                     const T* __restrict__ Bh, const T* __restrict__ gW,
-                                                     double* __restrict__ g5, T* __restrict__ gBcc) {
+                                                     const T* __restrict__ Bh, const T* __restrict__ W,
+                                                     const T* __restrict__ gW, double* __restrict__ g5,
+                                                     T* __restrict__ gBcc) {
   const Cell p = thread_cell(g);
   if (!p.ok) return;
   const long long N = g.N;
   const int c = p.c;
-  double h5[5], b[3];
+  double hy[4], b[3];
+  const bool pfl = at_p_floor<T>(g, W[4 * N + c]);
   if (HALF) {
 #pragma unroll
-    for (int f = 0; f < 5; ++f) h5[f] = Uh[f * N + c];
+    for (int f = 0; f < 4; ++f) hy[f] = Uh[f * N + c];
     b[0] = 0.5 * (to_d<T>(Bh[c + p.m[0]]) + to_d<T>(Bh[c]));
     b[1] = 0.5 * (to_d<T>(Bh[N + c + p.m[1]]) + to_d<T>(Bh[N + c]));
     b[2] = 0.5 * (to_d<T>(Bh[2 * N + c + p.m[2]]) + to_d<T>(Bh[2 * N + c]));
   } else {
 #pragma unroll
-    for (int f = 0; f < 5; ++f) h5[f] = U[f * N + c];
+    for (int f = 0; f < 4; ++f) hy[f] = U[f * N + c];
     b[0] = 0.5 * (U[5 * N + c + p.m[0]] + U[5 * N + c]);
     b[1] = 0.5 * (U[6 * N + c + p.m[1]] + U[6 * N + c]);
     b[2] = 0.5 * (U[7 * N + c + p.m[2]] + U[7 * N + c]);
@@ -626,7 +627,7 @@ __global__ void __launch_bounds__(BX* BY) k_adj_prim(Grid g, const double* __res
 #pragma unroll
     for (int f = 0; f < 8; ++f) gw8[f] = gW[f * N + c];
     float o5[5], gb[3];
-    prim_vjp_f32(g, h5[0], h5[1], h5[2], h5[3], h5[4], b, gw8, o5, gb);
+    prim_vjp_f32(g, hy[0], hy[1], hy[2], hy[3], pfl, b, gw8, o5, gb);
 #pragma unroll
     for (int f = 0; f < 5; ++f) g5[f * N + c] = f2d_bits(o5[f]);
     gBcc[c] = gb[0];
@@ -637,7 +638,7 @@ __global__ void __launch_bounds__(BX* BY) k_adj_prim(Grid g, const double* __res
 #pragma unroll
     for (int f = 0; f < 8; ++f) gw8[f] = to_d<T>(gW[f * N + c]);
     double o5[5], gb[3] = {0.0, 0.0, 0.0};
-    prim_vjp(g, h5[0], h5[1], h5[2], h5[3], h5[4], b, gw8, o5, gb);
+    prim_vjp(g, hy[0], hy[1], hy[2], hy[3], pfl, b, gw8, o5, gb);
 #pragma unroll
     for (int f = 0; f < 5; ++f) g5[f * N + c] = o5[f];
     gBcc[c] = from_d<T>(gb[0]);
@@ -690,7 +691,17 @@ __global__ void __launch_bounds__(BX* BY) k_fwd_half_keep(Grid g, const double* 
 #pragma unroll
   for (int f = 0; f < 5; ++f) Uh[f * N + c] = u5[f];
   const double bcc[3] = {0.5 * (bxm + bx), 0.5 * (bym + by), 0.5 * (bzm + bz)};
-  const PrimD pw = prim_core(g, u5[0], u5[1], u5[2], u5[3], u5[4], bcc);
+  PrimD pw = prim_core(g, u5[0], u5[1], u5[2], u5[3], u5[4], bcc);
+  if constexpr (std::is_same<T, float>::value) {
+    // the forward's floor decision (k_update_half recovers P by p_recover_f32),
+    // which the reverse reads off W: only the rounding of cells at the floor
+    const double bs[3] = {bxm + bx, bym + by, bzm + bz};
+    double t2, pe;
+    p_recover_f32(trcp<double>(pw.rho), u5[1], u5[2], u5[3], u5[4], bs, t2, pe);
+    const double pg = g.gm1 * pe;
+    if (!(pg > g.p_floor)) pw.p = g.p_floor;
+    else if (!(pw.p > g.p_floor)) pw.p = pg;
+  }
   T w8[8];
   store_w<T>(fields<8>(W, N), c, pw, w8);
 }
@@ -736,6 +747,7 @@ __global__ void __launch_bounds__(BX* BY) k_adj_cfl_argmax(Grid g, const T* __re
 constexpr int kCflThreads = 256;
 template <class T>  // (instantiated once per compute type's translation unit)
 __global__ void __launch_bounds__(kCflThreads) k_adj_cfl_term(Grid g, const double* __restrict__ U,
+                                                              const T* __restrict__ W,
                                                               const double* __restrict__ part, long long nparts,
                                                               const unsigned long long* __restrict__ rbits,
                                                               const unsigned long long* __restrict__ idx,
@@ -795,7 +807,7 @@ __global__ void __launch_bounds__(kCflThreads) k_adj_cfl_term(Grid g, const doub
   gw8[5 + (l + 1) % 3] = coef * dcf[3];
   gw8[5 + (l + 2) % 3] = coef * dcf[4];
   double o5[5], gb[3] = {0.0, 0.0, 0.0};
-  prim_vjp(g, r0, m[0], m[1], m[2], e, b, gw8, o5, gb);
+  prim_vjp(g, r0, m[0], m[1], m[2], at_p_floor<T>(g, W[4 * N + c]), b, gw8, o5, gb);
 #pragma unroll
   for (int f = 0; f < 5; ++f) gU[f * N + c] += o5[f];
 #pragma unroll
@@ -865,7 +877,7 @@ void AdjLaunch<T>::cfl_term(const Grid& g, const double* U, const T* W, const un
                             cudaStream_t s) {
     cudaMemsetAsync(idx, 0xff, sizeof(unsigned long long), s);
     k_adj_cfl_argmax<T><<<grid_of(g), dim3(BX, BY), 0, s>>>(g, W, rbits, idx);
-    k_adj_cfl_term<T><<<1, kCflThreads, 0, s>>>(g, U, part, nparts, rbits, idx, gU, out);
+    k_adj_cfl_term<T><<<1, kCflThreads, 0, s>>>(g, U, W, part, nparts, rbits, idx, gU, out);
   }
 template <class T>
 void AdjLaunch<T>::emf(const Grid& g, const T* W, const T* F, const T* gE, T* gF, T* gW, cudaStream_t s) {
@@ -946,12 +958,12 @@ void AdjLaunch<T>::recon(const Grid& g, int rc, int a, const T* W, const T* gWL,
     }
   }
 template <class T>
-void AdjLaunch<T>::prim(const Grid& g, bool half, const double* U, const double* Uh, const T* Bh, const T* gW, double* g5,
-                   T* gBcc, cudaStream_t s) {
+void AdjLaunch<T>::prim(const Grid& g, bool half, const double* U, const double* Uh, const T* Bh, const T* W,
+                        const T* gW, double* g5, T* gBcc, cudaStream_t s) {
     if (half)
-      k_adj_prim<T, true><<<grid_of(g), dim3(BX, BY), 0, s>>>(g, U, Uh, Bh, gW, g5, gBcc);
+      k_adj_prim<T, true><<<grid_of(g), dim3(BX, BY), 0, s>>>(g, U, Uh, Bh, W, gW, g5, gBcc);
     else
-      k_adj_prim<T, false><<<grid_of(g), dim3(BX, BY), 0, s>>>(g, U, Uh, Bh, gW, g5, gBcc);
+      k_adj_prim<T, false><<<grid_of(g), dim3(BX, BY), 0, s>>>(g, U, Uh, Bh, W, gW, g5, gBcc);
   }
 template <class T>
 void AdjLaunch<T>::faces_n(const Grid& g, const double* g5, const T* gBcc, const T* gBf, double* gU, cudaStream_t s) {

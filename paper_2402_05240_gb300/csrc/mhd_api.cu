@@ -504,7 +504,7 @@ int adjoint_step(mhd_ctx* c, const double* Un, double dt, const double* gUp, dou
     mhd::AdjLaunch<T>::recon(g, rc, a, b.Wh, b.gWL, b.gWR, b.gS, b.gW, ppmc_rev_scratch<T>(b, a, N), s);
   }
   // Step 5 (primitives of the half state, half update)
-  mhd::AdjLaunch<T>::prim(g, true, U, b.Uh, b.Bh, b.gW, b.g5, b.gBcc, s);
+  mhd::AdjLaunch<T>::prim(g, true, U, b.Uh, b.Bh, b.Wh, b.gW, b.g5, b.gBcc, s);
   // (the predictor edge fields, overwritten by Step 8's, again for the dt cotangent)
   if (cfl) Launch<T>::emf(g, b.Wn, b.Fn, b.Eh, s);
   mhd::AdjLaunch<T>::update(g, 1, 0.5 * dt, b.g5, nullptr, b.gBcc, b.gBf, gU, b.gF, b.gE, s, b.Fn, b.Eh, part1);
@@ -516,7 +516,7 @@ int adjoint_step(mhd_ctx* c, const double* Un, double dt, const double* gUp, dou
     mhd::AdjLaunch<T>::pcm_gather(g, a, b.gWL, b.gWR, b.gW, s);
   }
   // Step 1 (primitives of U^n) and the face cotangents
-  mhd::AdjLaunch<T>::prim(g, false, U, nullptr, nullptr, b.gW, b.g5, b.gBcc, s);
+  mhd::AdjLaunch<T>::prim(g, false, U, nullptr, nullptr, b.Wn, b.gW, b.g5, b.gBcc, s);
   mhd::AdjLaunch<T>::faces_n(g, b.g5, b.gBcc, b.gBf, gU, s);
   if (!cfl) return cuda_status();
   mhd::AdjLaunch<T>::cfl_term(g, U, b.Wn, c->dtbits, b.part, b.nparts, b.idx, gU, b.out, s);
@@ -544,7 +544,7 @@ int stage_recon_vjp(mhd_ctx* c, const double* U, int axis, int recon, const doub
   cudaMemsetAsync(b.gBf, 0, 3 * N * sizeof(T), s);
   cudaMemsetAsync(gU, 0, 8 * N * sizeof(double), s);
   mhd::AdjLaunch<T>::recon(g, recon, axis, b.Wn, b.gWL, b.gWR, b.gS, b.gW, ppmc_rev_scratch<T>(b, axis, N), s);
-  mhd::AdjLaunch<T>::prim(g, false, U, nullptr, nullptr, b.gW, b.g5, b.gBcc, s);
+  mhd::AdjLaunch<T>::prim(g, false, U, nullptr, nullptr, b.Wn, b.gW, b.g5, b.gBcc, s);
   mhd::AdjLaunch<T>::faces_n(g, b.g5, b.gBcc, b.gBf, gU, s);
   return cuda_status();
 }

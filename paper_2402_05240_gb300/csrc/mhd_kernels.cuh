@@ -191,11 +191,22 @@ template <class T> __device__ __forceinline__ T cell_inv_crossing(const Grid& g,
   return best;
 }
 
+// Gas-pressure recovery of the double and float-pair modes: mv = m.v, bb =
+// |B_cc|^2 and pe = E - mv/2 - bb/2, so that P = (gamma - 1) pe.  Written with
+// explicit multiply-adds, so the forward step and its reverse (which repeats
+// the floor decision) evaluate it alike whatever surrounds it.
+__device__ __forceinline__ void p_recover(const double* m, const double* v, double e, const double* b, double& mv,
+                                          double& bb, double& pe) {
+  mv = fma(m[2], v[2], fma(m[0], v[0], m[1] * v[1]));
+  bb = fma(b[2], b[2], fma(b[0], b[0], b[1] * b[1]));
+  pe = fma(-0.5, bb, fma(-0.5, mv, e));
+}
+
 // primitives from a double state of one cell: rho' = max(rho, floor),
-// v = m / rho', P' = max((gamma-1)(E - (m.v + |B_cc|^2)/2), floor).  t2 = m.v +
-// |B_cc|^2 and pg, the pressure before the floor, serve the floor reset.
+// v = m / rho', P' = max((gamma-1)(E - m.v/2 - |B_cc|^2/2), floor).  mv, bb
+// (p_recover) and pg, the pressure before the floor, serve the floor reset.
 __device__ __forceinline__ PrimD prim_core_ir(const Grid& g, double rho, double ir, double m0, double m1, double m2,
-                                              double e, const double* b, double& t2, double& pg) {
+                                              double e, const double* b, double& mv, double& bb, double& pg) {
   PrimD w;
   w.b[0] = b[0];
   w.b[1] = b[1];
@@ -204,8 +215,10 @@ __device__ __forceinline__ PrimD prim_core_ir(const Grid& g, double rho, double 
   w.v[0] = m0 * ir;
   w.v[1] = m1 * ir;
   w.v[2] = m2 * ir;
-  t2 = (m0 * w.v[0] + m1 * w.v[1] + m2 * w.v[2]) + (b[0] * b[0] + b[1] * b[1] + b[2] * b[2]);
-  pg = g.gm1 * (e - 0.5 * t2);
+  const double m[3] = {m0, m1, m2};
+  double pe;
+  p_recover(m, w.v, e, b, mv, bb, pe);
+  pg = g.gm1 * pe;
   w.p = max_pos<double>(pg, g.p_floor);
   return w;
 }
@@ -213,8 +226,8 @@ __device__ __forceinline__ PrimD prim_core_ir(const Grid& g, double rho, double 
 __device__ __forceinline__ PrimD prim_core(const Grid& g, double r, double m0, double m1, double m2, double e,
                                            const double* b) {
   const double rho = max_pos<double>(r, g.rho_floor);
-  double t2, pg;
-  return prim_core_ir(g, rho, trcp<double>(rho), m0, m1, m2, e, b, t2, pg);
+  double mv, bb, pg;
+  return prim_core_ir(g, rho, trcp<double>(rho), m0, m1, m2, e, b, mv, bb, pg);
 }
 
 // Cell-centred reference electric field E = -(v x B_cc) of one cell (Sec. 2.2
@@ -250,11 +263,11 @@ template <class T> __device__ __forceinline__ void store_w(const Fields<T, 8>& W
   for (int f = 0; f < 8; ++f) W.f[f][c] = w8[f];
 }
 
-// The energy that puts the pressure at its floor (t2 = m.v + |B_cc|^2).  A call,
-// made only in warps where a cell is floored: inlined, every warp issues its
-// FP64 instructions, two of the 14 to 20 of the primitive kernels.
-static __device__ __noinline__ double floored_energy(double p_floor, double igm1, double t2) {
-  return p_floor * igm1 + 0.5 * t2;
+// The energy that puts the pressure at its floor (x + y = m.v + |B_cc|^2).  A
+// call, made only in warps where a cell is floored: inlined, every warp issues
+// its FP64 instructions, two of the 14 to 20 of the primitive kernels.
+static __device__ __noinline__ double floored_energy(double p_floor, double igm1, double x, double y) {
+  return fma(0.5, y, p_floor * igm1 + 0.5 * x);
 }
 
 // FP32-bulk gas-pressure recovery in double: t2 = |m|^2 / rho' + |B_cc|^2
@@ -297,13 +310,14 @@ __device__ __forceinline__ void prim_store_f32(const Grid& g, const Fields<float
   for (int f = 0; f < 8; ++f) W.f[f][c] = w8[f];
 }
 
-// end-of-step pressure floor of one cell (floors null: none); in: an interior cell
+// end-of-step pressure floor of one cell (floors null: none); in: an interior
+// cell; x + y = m.v + |B_cc|^2
 __device__ __forceinline__ void floor_energy(const Grid& g, const Fields<double, 8>& U, int c,
-                                             unsigned long long* floors, bool in, double pg, double t2) {
+                                             unsigned long long* floors, bool in, double pg, double x, double y) {
   const bool low = floors && lt_pos<double>(pg, g.p_floor);
   if (__any_sync(__activemask(), low)) {
     if (low) {
-      U.f[4][c] = floored_energy(g.p_floor, g.igm1, t2);
+      U.f[4][c] = floored_energy(g.p_floor, g.igm1, x, y);
       if (in) atomicAdd(&floors[1], 1ull);
     }
   }
@@ -348,13 +362,13 @@ __global__ void __launch_bounds__(BX* BY) k_prim(Grid g, Fields<double, 8> U, Fi
       double t2, pg;
       prim_store_f32(g, W, c, rho, ir, m0, m1, m2, e, bs, w8, t2, pg);
       store_ref<T>(Er, c, w8);
-      floor_energy(g, U, c, floors, in, pg, t2);
+      floor_energy(g, U, c, floors, in, pg, t2, 0.0);
       if (dtbits && in) inv = cell_inv_crossing<T>(g, w8);
     } else {
       const double b[3] = {half<double>(b0m + b0p), half<double>(b1m + b1p), half<double>(b2m + b2p)};
-      double t2, pg;
-      const PrimD pw = prim_core_ir(g, rho, ir, m0, m1, m2, e, b, t2, pg);
-      floor_energy(g, U, c, floors, in, pg, t2);
+      double mv, bb, pg;
+      const PrimD pw = prim_core_ir(g, rho, ir, m0, m1, m2, e, b, mv, bb, pg);
+      floor_energy(g, U, c, floors, in, pg, mv, bb);
       store_w<T>(W, c, pw, w8);
       store_ref<T>(Er, c, w8);
       if (dtbits && in) {

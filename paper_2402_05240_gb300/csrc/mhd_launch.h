@@ -109,8 +109,8 @@ template <class T> struct AdjLaunch {
   // for the other reconstructions)
   static void recon(const Grid& g, int rc, int a, const T* W, const T* gWL, const T* gWR, T* S, T* gW,
                     const Fields<T, kPpmcRevFields>& X, cudaStream_t s);
-  static void prim(const Grid& g, bool half, const double* U, const double* Uh, const T* Bh, const T* gW, double* g5,
-                   T* gBcc, cudaStream_t s);
+  static void prim(const Grid& g, bool half, const double* U, const double* Uh, const T* Bh, const T* W, const T* gW,
+                   double* g5, T* gBcc, cudaStream_t s);
   static void faces_n(const Grid& g, const double* g5, const T* gBcc, const T* gBf, double* gU, cudaStream_t s);
   static void fwd_half_keep(const Grid& g, const double* U, const T* F, const T* E, double dt, T* W, T* Bh, double* Uh,
                             cudaStream_t s);
