@@ -433,7 +433,7 @@ __device__ void plmc_vjp(T gamma, T rho_floor, T p_floor, const T* wm, const T* 
     if (pos_prod<T>(aL[q], aR[q])) {
       // the selections of the forward min_abs(min_abs(2 aL, 2 aR), min_abs(aC, aG)),
       // ties to the second operand
-      const T c0 = fabs(twice<T>(aL[q])), c1 = fabs(twice<T>(aR[q])), c2 = fabs(aC[q]), c3 = fabs(aG[q]);
+      const T c0 = fabs(twice_n<T>(aL[q])), c1 = fabs(twice_n<T>(aR[q])), c2 = fabs(aC[q]), c3 = fabs(aG[q]);
       const int s01 = nonneg_lt<T>(c0, c1) ? 0 : 1;
       const T m01 = s01 == 0 ? c0 : c1;
       const int s23 = nonneg_lt<T>(c2, c3) ? 2 : 3;

@@ -139,14 +139,30 @@ template <> __device__ __forceinline__ double neg<double>(double x) {
 // intrinsics: written on the 64-bit pattern the compiler recognises them as
 // negations and absolute values and, where they feed a selection, issues them
 // as additions on the FP64 pipe.)
-// Scalings by 2, 4 and 1/2.  Double: on the bit pattern.  twice() serves the
-// limiters (finite normal operands or zeros, no overflow); half() is exact for
-// every operand but odd subnormals (cut by half the smallest one); quad()
+// Scalings by 2, 4 and 1/2.  Double: on the bit pattern.  twice() is the IEEE
+// product for every operand (the reverse doubles cotangents, which may be
+// infinite or NaN); half() is exact for every operand but odd subnormals (cut
+// by half the smallest one); quad()
 // falls back to the multiplication, executed only in warps where a lane needs
 // it, where operand or result is not normal.
 template <class T> __device__ __forceinline__ T twice(T x) { return T(2) * x; }
 template <> __device__ __forceinline__ df twice<df>(df x) { return df(2.0f * x.hi, 2.0f * x.lo); }
 template <> __device__ __forceinline__ double twice<double>(double v) {
+  const int hi = __double2hiint(v), lo = __double2loint(v), m = hi & 0x7fffffff;
+  const bool small = m < 0x00100000;  // zero or subnormal
+  int rh = small ? (int)__funnelshift_l((unsigned)lo, (unsigned)m, 1) | (hi & (int)0x80000000) : hi + 0x00100000;
+  int rl = small ? (int)((unsigned)lo << 1) : lo;
+  if (m >= 0x7fe00000) {  // the result is an infinity, or v a NaN
+    rh = m >= 0x7ff00000 ? hi : (hi | 0x7ff00000) & (int)0xfff00000;
+    rl = m >= 0x7ff00000 ? lo : 0;
+  }
+  return __hiloint2double(rh, rl);
+}
+// twice_n: for the limiters' operands, zero or normal and without overflow.
+// (256^3, FP64, with twice() in its place: PLMC reconstruction 18.56 -> 18.79 ms,
+// PPMC 32.65 -> 32.86.)
+template <class T> __device__ __forceinline__ T twice_n(T x) { return twice<T>(x); }
+template <> __device__ __forceinline__ double twice_n<double>(double v) {
   const int hi = __double2hiint(v), lo = __double2loint(v);
   return __hiloint2double(((hi & 0x7fffffff) | lo) ? hi + 0x00100000 : hi, lo);
 }
@@ -285,6 +301,7 @@ template <class T> struct Ops {
   __device__ __forceinline__ T sqrt(T x) { return tsqrt<T>(x); }
   __device__ __forceinline__ T rsqrt(T x) { return trsqrt<T>(x); }
   __device__ __forceinline__ T quad(T x) { return mhd::quad<T>(x); }
+  __device__ __forceinline__ T twice(T x) { return mhd::twice<T>(x); }
   __device__ __forceinline__ auto mul(T a, T b) { return mulc<T>(a, b); }
 };
 struct TryValue {
@@ -307,6 +324,9 @@ template <> struct TryOps<double> {
     bad |= (b != 0) & ((unsigned long long)(b - (1LL << 52)) >= (0x7fdULL << 52) - (1ULL << 52));
     return __longlong_as_double(b ? b + (2LL << 52) : b);
   }
+  // (of a root or a product: below 2^1023, and not normal or zero only where
+  // bad is set already)
+  __device__ __forceinline__ double twice(double x) { return twice_n<double>(x); }
   __device__ __forceinline__ double mul(double a, double b) {
     const TryValue r = mul_try_call(a, b);
     bad |= r.bad != 0;
@@ -680,8 +700,8 @@ template <class T, class O> __device__ __forceinline__ void eig_build(O& o, T ga
   } else {
     const bool dpos = ge0<T>(D);
     const T sa = sd + absv<T>(D);
-    const T q = o.rsqrt(o.mul(twice<T>(sd), sa));
-    const T big = o.mul(sa, q), small = o.mul(o.mul(twice<T>(E.a), btn), q);
+    const T q = o.rsqrt(o.mul(o.twice(sd), sa));
+    const T big = o.mul(sa, q), small = o.mul(o.mul(o.twice(E.a), btn), q);
     E.af = dpos ? big : small;
     E.as = dpos ? small : big;
   }
@@ -865,7 +885,7 @@ template <class T, class O> __device__ __forceinline__ void van_leer7(O& o, cons
       // a product that underflows gives 0, also where 1/s would overflow
       const bool act = pos_prod<T>(dL[q], dR[q]);
       const T pr = dL[q] * dR[q];
-      const T g = twice<T>(pr) * o.rcp(act ? dL[q] + dR[q] : 1.0);
+      const T g = twice_n<T>(pr) * o.rcp(act ? dL[q] + dR[q] : 1.0);
       dG[q] = (act && !is0<T>(pr)) ? g : T(0);
     } else if constexpr (std::is_same<T, df>::value) {
       // the sign from the product's leading float: pos_prod<df> holds for a
@@ -905,7 +925,7 @@ __device__ __forceinline__ void plmc(O& o, T gamma, const T* wm, const T* w0, co
 #pragma unroll
   for (int q = 0; q < 7; ++q) {
     if (pos_prod<T>(aL[q], aR[q])) {
-      const T m = min_abs<T>(min_abs<T>(twice<T>(aL[q]), twice<T>(aR[q])), min_abs<T>(aC[q], aG[q]));
+      const T m = min_abs<T>(min_abs<T>(twice_n<T>(aL[q]), twice_n<T>(aR[q])), min_abs<T>(aC[q], aG[q]));
       am[q] = with_sign<T>(aC[q], m);
     } else {
       am[q] = T(0);
@@ -1005,8 +1025,8 @@ template <class T> __device__ __forceinline__ void ppm_one_wide(const T* q, T& q
     }
   } else {
     const T m0 = qm;
-    if (abs_ge_twice<T>(qm, qp)) qm = neg<T>(twice<T>(qp));
-    if (abs_ge_twice<T>(qp, m0)) qp = neg<T>(twice<T>(m0));
+    if (abs_ge_twice<T>(qm, qp)) qm = neg<T>(twice_n<T>(qp));
+    if (abs_ge_twice<T>(qp, m0)) qp = neg<T>(twice_n<T>(m0));
   }
 }
 
@@ -1059,8 +1079,8 @@ template <class T> __device__ __forceinline__ void ppm_one(const T* q, T& qm, T&
     qp = r * qp;
   } else {
     const T m0 = qm;
-    if (abs_ge_twice<T>(qm, qp)) qm = neg<T>(twice<T>(qp));
-    if (abs_ge_twice<T>(qp, m0)) qp = neg<T>(twice<T>(m0));
+    if (abs_ge_twice<T>(qm, qp)) qm = neg<T>(twice_n<T>(qp));
+    if (abs_ge_twice<T>(qp, m0)) qp = neg<T>(twice_n<T>(m0));
   }
 }
 

@@ -144,3 +144,81 @@ int main() {
 def test_plmc_with_tiny_differences(tmp_path, typ):
     """Differences whose product underflows leave van Leer's mean at zero."""
     assert compile_and_run(tmp_path, TINY_DIFFERENCES.replace("TYPE", typ)) == ["0"]
+
+
+DOUBLING = r"""
+int main() {
+  long bad = 0;
+  for (double x : values(60)) bad += !same(twice<double>(x), 2.0 * x);
+  printf("%ld\n", bad);
+}
+"""
+
+
+def test_doubling_is_the_ieee_one(tmp_path):
+    assert compile_and_run(tmp_path, DOUBLING) == ["0"]
+
+
+NONFINITE = r"""
+// outputs of a reverse function that respond to cotangent q have to be
+// non-finite where that cotangent is
+template <class F> static long lost(int nin, int nout, F f) {
+  long bad = 0;
+  std::vector<double> g(nin), o(nout), r(nout);
+  for (int q = 0; q < nin; ++q)
+    for (double x : {std::numeric_limits<double>::infinity(), std::numeric_limits<double>::quiet_NaN()}) {
+      for (int k = 0; k < nin; ++k) g[k] = k == q ? 1.0 : 0.0;
+      f(g.data(), o.data());
+      for (int k = 0; k < nin; ++k) g[k] = k == q ? x : 0.1 + k;
+      f(g.data(), r.data());
+      for (int k = 0; k < nout; ++k) bad += o[k] != 0.0 && std::isfinite(r[k]);
+    }
+  return bad;
+}
+int main() {
+  typedef TYPE T;
+  std::mt19937_64 rng(5);
+  std::normal_distribution<double> n;
+  long hlld = 0, ppmc = 0, plmc = 0;
+  for (int it = 0; it < 300; ++it) {
+    double w[5][7], bn = n(rng);
+    const double base[7] = {exp(0.3 * n(rng)), (it % 3) * n(rng), n(rng), n(rng), exp(0.3 * n(rng)), 0.5 * n(rng), 0.5 * n(rng)};
+    double slope[7];
+    for (double& s : slope) s = 0.05 * n(rng);
+    for (int m = 0; m < 5; ++m)
+      for (int q = 0; q < 7; ++q) w[m][q] = base[q] * (1.0 + 0.01 * n(rng)) + slope[q] * (m - 2);
+    T W[5][7];
+    for (int m = 0; m < 5; ++m)
+      for (int q = 0; q < 7; ++q) W[m][q] = T(w[m][q]);
+    hlld += lost(7, 15, [&](const double* g, double* o) {
+      T gf[7], a[7], b[7], c = T(0);
+      for (int q = 0; q < 7; ++q) gf[q] = T(g[q]), a[q] = b[q] = T(0);
+      hlld_vjp<T>(T(5.0 / 3.0), W[1], W[2], T(bn), gf, a, b, c);
+      for (int q = 0; q < 7; ++q) o[q] = to_d<T>(a[q]), o[7 + q] = to_d<T>(b[q]);
+      o[14] = to_d<T>(c);
+    });
+    ppmc += lost(14, 36, [&](const double* g, double* o) {
+      T gl[7], gr[7], G[5][7], c = T(0);
+      for (int q = 0; q < 7; ++q) gl[q] = T(g[q]), gr[q] = T(g[7 + q]);
+      for (int q = 0; q < 35; ++q) G[q / 7][q % 7] = T(0);
+      ppmc_vjp<T>(T(5.0 / 3.0), T(1e-20), T(1e-20), [&](int m, T* v) { for (int q = 0; q < 7; ++q) v[q] = W[m][q]; }, T(bn),
+                  gl, gr, [&](int m, const T* v) { for (int q = 0; q < 7; ++q) G[m][q] = v[q]; }, G[2], c);
+      for (int q = 0; q < 35; ++q) o[q] = to_d<T>(G[q / 7][q % 7]);
+      o[35] = to_d<T>(c);
+    });
+    plmc += lost(14, 22, [&](const double* g, double* o) {
+      T gl[7], gr[7], G[3][7], c = T(0);
+      for (int q = 0; q < 7; ++q) gl[q] = T(g[q]), gr[q] = T(g[7 + q]), G[0][q] = G[1][q] = G[2][q] = T(0);
+      plmc_vjp<T>(T(5.0 / 3.0), T(1e-20), T(1e-20), W[1], W[2], W[3], T(bn), gl, gr, G[0], G[1], G[2], c);
+      for (int q = 0; q < 21; ++q) o[q] = to_d<T>(G[q / 7][q % 7]);
+      o[21] = to_d<T>(c);
+    });
+  }
+  printf("%ld %ld %ld\n", hlld, ppmc, plmc);
+}
+"""
+
+
+@pytest.mark.parametrize("typ", ["double", "df"])
+def test_nonfinite_cotangents_reach_the_gradient(tmp_path, typ):
+    assert compile_and_run(tmp_path, NONFINITE.replace("TYPE", typ)) == ["0", "0", "0"]
