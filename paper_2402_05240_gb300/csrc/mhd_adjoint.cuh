@@ -1801,7 +1801,7 @@ __device__ void hlld_vjp(T gamma, const T* wl, const T* wr, T bn, const T* gf, T
 // again: where the kinetic and magnetic energy exceed the floor by 1 / eps, as in
 // every cell that a floor has just reset, it is the sign of a rounding error.
 template <class T> __device__ __forceinline__ bool at_p_floor(const Grid& g, T p) {
-  return !(p > from_d<T>(g.p_floor));
+  return !(p > nearest<T>(g.p_floor));  // (converted as the forward's store_w does)
 }
 __device__ __forceinline__ void prim_vjp(const Grid& g, double r, double m0, double m1, double m2, bool pfl,
                                          const double* b, const double* gW, double* g5, double* gb) {

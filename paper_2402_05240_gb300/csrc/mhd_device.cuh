@@ -238,6 +238,9 @@ template <class T> __device__ __forceinline__ T from_d(double x);
 template <> __device__ __forceinline__ double from_d<double>(double x) { return x; }
 template <> __device__ __forceinline__ float from_d<float>(double x) { return d2f_bits(x); }
 template <> __device__ __forceinline__ df from_d<df>(double x) { return df(x); }
+// (float pairs: with the longer low part)
+template <class T> __device__ __forceinline__ T nearest(double x) { return from_d<T>(x); }
+template <> __device__ __forceinline__ df nearest<df>(double x) { return df_nearest(x); }
 
 // Exact<T>: the full update widens each flux and edge value to double before
 // differencing (a difference of two floats is exact in double).  df values

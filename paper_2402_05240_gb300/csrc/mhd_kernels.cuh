@@ -247,14 +247,14 @@ template <class T> __device__ __forceinline__ void store_ref(const Fields<T, 3>&
 }
 
 template <class T> __device__ __forceinline__ void prim_to_w8(const PrimD& p, T* w8) {
-  w8[0] = from_d<T>(p.rho);
-  w8[1] = from_d<T>(p.v[0]);
-  w8[2] = from_d<T>(p.v[1]);
-  w8[3] = from_d<T>(p.v[2]);
-  w8[4] = from_d<T>(p.p);
-  w8[5] = from_d<T>(p.b[0]);
-  w8[6] = from_d<T>(p.b[1]);
-  w8[7] = from_d<T>(p.b[2]);
+  w8[0] = nearest<T>(p.rho);
+  w8[1] = nearest<T>(p.v[0]);
+  w8[2] = nearest<T>(p.v[1]);
+  w8[3] = nearest<T>(p.v[2]);
+  w8[4] = nearest<T>(p.p);
+  w8[5] = nearest<T>(p.b[0]);
+  w8[6] = nearest<T>(p.b[1]);
+  w8[7] = nearest<T>(p.b[2]);
 }
 
 template <class T> __device__ __forceinline__ void store_w(const Fields<T, 8>& W, int c, const PrimD& p, T* w8) {

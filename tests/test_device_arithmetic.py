@@ -222,3 +222,35 @@ int main() {
 @pytest.mark.parametrize("typ", ["double", "df"])
 def test_nonfinite_cotangents_reach_the_gradient(tmp_path, typ):
     assert compile_and_run(tmp_path, NONFINITE.replace("TYPE", typ)) == ["0", "0", "0"]
+
+
+CONVERSION = r"""
+int main() {
+  std::mt19937_64 g(7);
+  const uint64_t all = (1ull << 52) - 1;
+  long bad = 0;
+  for (int i = 0; i < 400000; ++i) {
+    uint64_t f = g() & all;
+    if (i % 4 == 1) f = ((f >> 29) << 29) + (1ull << 28) + (g() % 3) - 1;  // about halfway between two floats
+    if (i % 4 == 2) f = all - (g() & 0xffffffff);                          // hi carries into the exponent
+    const int e = i % 4 == 3 ? 944 + (int)(g() % 2) : 944 + (int)(g() % 207);
+    if (e == 1150 && f > all - (1ull << 30)) continue;  // rounds to 2^128
+    const double x = word_cast<double>(((uint64_t)e << 52) | f) * (g() & 1 ? 1.0 : -1.0);
+    const df d = nearest<df>(x);
+    bad += !(fabsl(((long double)d.hi - (long double)x) + (long double)d.lo) <= 0x1p-48L * fabsl((long double)x));
+    bad += fabs(x - d.hi) != fabs(x - (float)x);       // normalised: hi is x to nearest
+  }
+  for (double x : values(4)) {
+    const df d = nearest<df>(x), t = df_from_double(x);
+    const bool tiny = fabs(x) < 0x1p-79, huge = !(fabs(x) < 0x1p127);
+    if (tiny) bad += !(fabs((double)d.hi - x) <= fabs(x) * 0x1p-24 + 0x1p-126) + !(fabsf(d.lo) <= 0x1p-100f);
+    if (huge) bad += !(d.hi == t.hi || (d.hi != d.hi && t.hi != t.hi) || std::isinf(d.hi));
+  }
+  printf("%ld\n", bad);
+}
+"""
+
+
+def test_float_pairs_of_the_primitives(tmp_path):
+    """Within 2^-48 of the double (from_d<df> keeps 2^-47)."""
+    assert compile_and_run(tmp_path, CONVERSION) == ["0"]
