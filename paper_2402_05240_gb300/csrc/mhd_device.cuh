@@ -297,7 +297,7 @@ template <class T> __device__ __forceinline__ auto mulc(T a, T b) {
 // spill registers and outgrow the instruction cache (PPMC with the projections'
 // products 45.8 ms inlined, 33.2 ms as calls; Riemann kernels with 38 products
 // 10.2 and 8.7 ms).  Measured at 256^3, FP64: Riemann kernels 10.9 -> 8.7 ms, PLMC
-// reconstruction 23.9 -> 18.6 ms, PPMC 41.4 -> 32.6 ms.
+// reconstruction 23.9 -> 18.4 ms, PPMC 41.4 -> 32.5 ms.
 template <class T> struct Ops {
   static constexpr bool bad = false;
   __device__ __forceinline__ T rcp(T x) { return trcp<T>(x); }
@@ -803,6 +803,43 @@ template <class T> __device__ __forceinline__ void eig_left(const Eig<T>& E, con
   eig_left<T>(o, E, C, dw, q);
 }
 
+// The eigensystem and its coefficients.  A cell whose operands leave the range
+// of the integer-pipe functions here (a field below 1e-154) has these evaluated
+// again out of line, and not its whole reconstruction.  Measured at 128^3 (FP64,
+// fields of 1e-160 everywhere), ms per step with the whole cell evaluated again,
+// and as here: PLMC 10.69 and 9.55 (library functions throughout: 10.59), PPMC
+// 13.15 and 11.21 (12.52); with fields of order one 5.93 and 5.85, 7.28 and 7.24.
+template <class T> struct EigSystem {
+  Eig<T> E;
+  EigCoef<T> C;
+};
+template <class T> __device__ __noinline__ void eig_again(T gamma, const T* w, T bn, EigSystem<T>& S) {
+  Ops<T> o;
+  eig_build<T>(o, gamma, w, bn, S.E);
+  S.C = eig_coef<T>(o, S.E);
+}
+// (with a range test of its own: o's may be set already)
+template <class T, class O>
+__device__ __forceinline__ EigCoef<T> eig_system(const O&, T gamma, const T* w, T bn, Eig<T>& E) {
+  O o;
+  eig_build<T>(o, gamma, w, bn, E);
+  EigCoef<T> C = eig_coef<T>(o, E);
+  if constexpr (std::is_same<O, TryOps<double>>::value) {
+    if (__any_sync(__activemask(), o.bad)) {
+      if (o.bad) {
+        T a[7];
+#pragma unroll
+        for (int q = 0; q < 7; ++q) a[q] = w[q];
+        EigSystem<T> S;
+        eig_again<T>(gamma, a, bn, S);
+        E = S.E;
+        C = S.C;
+      }
+    }
+  }
+  return C;
+}
+
 // primitive increments dw = R q
 template <class T> __device__ __forceinline__ void eig_right(const Eig<T>& E, const T* q, T* dw) {
   const T fp = q[0] + q[6], fm = q[0] - q[6];
@@ -915,9 +952,8 @@ __device__ __forceinline__ void plmc(O& o, T gamma, const T* wm, const T* w0, co
   }
   van_leer7<T>(o, dL, dR, dG);
   Eig<T> E;
-  eig_build<T>(o, gamma, w0, bn, E);
+  const EigCoef<T> C = eig_system<T>(o, gamma, w0, bn, E);
   T aL[7], aR[7], aC[7], aG[7], am[7], dW[7];
-  const EigCoef<T> C = eig_coef<T>(o, E);
   eig_left<T>(o, E, C, dL, aL);
   eig_left<T>(o, E, C, dR, aR);
   eig_left<T>(o, E, C, dG, aG);
@@ -1104,8 +1140,7 @@ template <class T> __device__ __noinline__ LimitedPair<T> ppm_one_call(T a, T b,
 template <class T, class O>
 __device__ __forceinline__ void ppmc(O& o, T gamma, const T (*w)[7], T bn, T* wl, T* wr) {
   Eig<T> E;
-  eig_build<T>(o, gamma, w[2], bn, E);
-  const EigCoef<T> C = eig_coef<T>(o, E);
+  const EigCoef<T> C = eig_system<T>(o, gamma, w[2], bn, E);
   T qs[5][7];
 #pragma unroll
   for (int m = 0; m < 5; ++m) {

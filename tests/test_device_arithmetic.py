@@ -254,3 +254,52 @@ int main() {
 def test_float_pairs_of_the_primitives(tmp_path):
     """Within 2^-48 of the double (from_d<df> keeps 2^-47)."""
     assert compile_and_run(tmp_path, CONVERSION) == ["0"]
+
+
+FALLBACK = r"""
+static long used = 0;
+int main() {
+  std::mt19937_64 g(23);
+  std::normal_distribution<double> n;
+  std::uniform_real_distribution<double> u;
+  long plm = 0, ppm = 0, hl = 0;
+  for (int it = 0; it < 40000; ++it) {
+    double w[5][7], scale[7], bn = n(g);
+    // components and differences of every size, zeros among them
+    auto tiny = [&] { return it % 4 == 0 ? 1.0 : u(g) < 0.2 ? 0.0 : std::pow(10.0, -330.0 * u(g)); };
+    const double base[7] = {exp(n(g)), n(g), n(g), n(g), exp(n(g)), n(g), n(g)};
+    for (double& s : scale) s = tiny();
+    bn *= tiny();
+    const double size[7] = {1.0, scale[1], scale[2], scale[3], 1.0, scale[5], scale[6]};
+    for (int m = 0; m < 5; ++m)
+      for (int q = 0; q < 7; ++q) w[m][q] = size[q] * base[q] * (1.0 + 0.05 * scale[(q + 3) % 7] * n(g));
+    double a[4][7], b[4][7];
+    {
+      TryOps<double> o;
+      plmc<double>(o, 5.0 / 3.0, w[1], w[2], w[3], bn, a[0], a[1]);
+      Ops<double> c;
+      plmc<double>(c, 5.0 / 3.0, w[1], w[2], w[3], bn, b[0], b[1]);
+      used += o.bad;
+      for (int k = 0; k < 14; ++k) plm += !o.bad && !same(a[k / 7][k % 7], b[k / 7][k % 7]);
+    }
+    {
+      TryOps<double> o;
+      ppmc<double>(o, 5.0 / 3.0, w, bn, a[0], a[1]);
+      Ops<double> c;
+      ppmc<double>(c, 5.0 / 3.0, w, bn, b[0], b[1]);
+      used += o.bad;
+      for (int k = 0; k < 14; ++k) ppm += !o.bad && !same(a[k / 7][k % 7], b[k / 7][k % 7]);
+    }
+    hlld<double>(5.0 / 3.0, 1.5, w[1], w[2], bn, a[2]);
+    Ops<double> c;
+    hlld_diff<double>(c, 5.0 / 3.0, 1.5, w[1], w[2], bn, b[2]);
+    for (int k = 0; k < 7; ++k) hl += !same(a[2][k], b[2][k]);
+  }
+  printf("%ld %ld %ld %d\n", plm, ppm, hl, used > 1000);
+}
+"""
+
+
+def test_cells_out_of_range_are_flagged(tmp_path):
+    """What the range tests let pass equals the complete functions, bit for bit."""
+    assert compile_and_run(tmp_path, FALLBACK, flags=("-ffp-contract=off",)) == ["0", "0", "0", "1"]
