@@ -141,8 +141,8 @@ template <> __device__ __forceinline__ double neg<double>(double x) {
 // as additions on the FP64 pipe.)
 // Scalings by 2, 4 and 1/2.  Double: on the bit pattern.  twice() is the IEEE
 // product for every operand (the reverse doubles cotangents, which may be
-// infinite or NaN); half() is exact for every operand but odd subnormals (cut
-// by half the smallest one); quad()
+// infinite or NaN); half() and quarter() cut results below 2^-1022 to a
+// multiple of the smallest subnormal and are exact otherwise; quad()
 // falls back to the multiplication, executed only in warps where a lane needs
 // it, where operand or result is not normal.
 template <class T> __device__ __forceinline__ T twice(T x) { return T(2) * x; }
@@ -213,8 +213,10 @@ template <> __device__ __forceinline__ df quarter<df>(df x) { return df(0.25f * 
 template <> __device__ __forceinline__ double quarter<double>(double x) {
   const int hi = __double2hiint(x), lo = __double2loint(x), m = hi & 0x7fffffff;
   const bool small = m < 0x00300000;  // operand or result not normal
-  const int rl = small ? (int)__funnelshift_r((unsigned)lo, (unsigned)m, 2) : lo;
-  const int rh = small ? (m >> 2) | (hi & (int)0x80000000) : hi - 0x00200000;
+  // (exponent field 2: down to 1, whose significand stands as a subnormal's does)
+  const int low = m < 0x00200000 ? m : m - 0x00100000, sh = m < 0x00200000 ? 2 : 1;
+  const int rl = small ? (int)__funnelshift_r((unsigned)lo, (unsigned)low, sh) : lo;
+  const int rh = small ? (low >> sh) | (hi & (int)0x80000000) : hi - 0x00200000;
   return __hiloint2double(m >= 0x7ff00000 ? hi : rh, rl);
 }
 // s x for s = +-1 (a sign flip for double and float pairs)

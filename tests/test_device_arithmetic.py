@@ -159,6 +159,25 @@ def test_doubling_is_the_ieee_one(tmp_path):
     assert compile_and_run(tmp_path, DOUBLING) == ["0"]
 
 
+SCALINGS = r"""
+int main() {
+  long h = 0, qt = 0, qd = 0;
+  for (double x : values(60)) {
+    // (results below 2^-1022 are cut, not rounded: the largest would round to it)
+    auto off = [](double r, double ref) { return fabs(ref) <= 0x1p-1022 ? !(fabs(r - ref) <= 0x1p-1074) : !same(r, ref); };
+    h += off(half<double>(x), 0.5 * x);
+    qt += off(quarter<double>(x), 0.25 * x);
+    qd += !same(quad<double>(x), 4.0 * x);
+  }
+  printf("%ld %ld %ld\n", h, qt, qd);
+}
+"""
+
+
+def test_scalings_at_the_ends_of_the_range(tmp_path):
+    assert compile_and_run(tmp_path, SCALINGS) == ["0", "0", "0"]
+
+
 NONFINITE = r"""
 // outputs of a reverse function that respond to cotangent q have to be
 // non-finite where that cotangent is
