@@ -207,7 +207,7 @@ template <> __device__ __forceinline__ double pick<double>(bool c, double a, dou
   return r;
 }
 #endif
-// x / 4; as half()
+// x / 4; as half() (edge fields, and |B_cc|^2 of the FP32-bulk pressure)
 template <class T> __device__ __forceinline__ T quarter(T x) { return T(0.25) * x; }
 template <> __device__ __forceinline__ df quarter<df>(df x) { return df(0.25f * x.hi, 0.25f * x.lo); }
 template <> __device__ __forceinline__ double quarter<double>(double x) {

@@ -20,8 +20,11 @@ inline long long cell_blocks(int nx, int ny, int nz) {
 // once (28 more words per cell).  Measured per PPMC step, three launches /
 // one, at 16^3, 32^3, 64^3, 96^3, 128^3, 160^3: FP32-bulk 75 / 47, 78 / 55,
 // 170 / 143, 415 / 388, 857 / 834, 1562 / 1551 us; FP64 182 / 113, 266 / 238,
-// 1419 / 1355, 4352 / 4276, 9957 / 9877, 19085 / 19005 us.  The line is at
-// 128^3, where the gain falls below 3 % and the words pass 0.5 GB.
+// 1419 / 1355, 4352 / 4276, 9957 / 9877, 19085 / 19005 us; float pairs at 32^3 and
+// 64^3 129 / 114 and 461 / 453 us.  The line is at 128^3, one for all types,
+// where the words pass 0.5 GB in double and the FP32-bulk gain falls below 3 %
+// (FP64 passes 3 % between 64^3 and 96^3 and gains 0.8 % at 128^3).  A context that
+// finds no room for the words runs one launch per axis (mhd_init).
 constexpr long long kFuseBlocks = 16384;
 inline bool fuse_axes(int nx, int ny, int nz) {
   return cell_blocks(nx, ny, nz) <= kFuseBlocks && nz <= 65535 / 3;
