@@ -629,11 +629,8 @@ template <class T> __device__ __forceinline__ void ppm_one_vjp_wide(const T* q, 
   gq[4] = g2p1 - c1 * gp;
 }
 
-template <class T> __device__ void ppm_one_vjp(const T* q, T gqm, T gqp, T* gq) {
-  if constexpr (sizeof(T) != 4) {
-    ppm_one_vjp_wide<T>(q, gqm, gqp, gq);
-    return;
-  }
+// (float)
+template <class T> __device__ void ppm_one_vjp_narrow(const T* q, T gqm, T gqp, T* gq) {
   const T c7 = from_d<T>(7.0 / 12.0), c1 = from_d<T>(1.0 / 12.0), c6 = from_d<T>(1.0 / 6.0);
   // forward, recording the branches
   T qm = c7 * (q[1] + q[2]) - c1 * (q[0] + q[3]);
@@ -759,6 +756,11 @@ template <class T> __device__ void ppm_one_vjp(const T* q, T gqm, T gqp, T* gq) 
   gq[3] += g20 - T(2) * g2p1;
   gq[4] += g2p1;
   gq[2] += gq2;
+}
+
+template <class T> __device__ __forceinline__ void ppm_one_vjp(const T* q, T gqm, T gqp, T* gq) {
+  if constexpr (sizeof(T) != 4) ppm_one_vjp_wide<T>(q, gqm, gqp, gq);
+  else ppm_one_vjp_narrow<T>(q, gqm, gqp, gq);
 }
 
 // (double and float pairs: a call with its operands in registers)
@@ -1411,16 +1413,9 @@ __device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, cons
   gbn += g_bn;
 }
 
-// Reverse of hlld(): gf = cotangent of the 7 flux components; accumulates
-// gwl[7], gwr[7] and gbn.  Follows the region selection, the degenerate
-// switches and the outer-speed selections of the forward solver.
+// (float: the reverse of hlld_jump)
 template <class T>
-__device__ void hlld_vjp(T gamma, const T* wl, const T* wr, T bn, const T* gf, T* gwl, T* gwr, T& gbn) {
-  const T gm1i = trcp<T>(gamma - T(1));
-  if constexpr (sizeof(T) != 4) {
-    hlld_diff_vjp<T>(gamma, gm1i, wl, wr, bn, gf, gwl, gwr, gbn);
-    return;
-  }
+__device__ void hlld_jump_vjp(T gamma, T gm1i, const T* wl, const T* wr, T bn, const T* gf, T* gwl, T* gwr, T& gbn) {
   const T bn2 = bn * bn;
   T eL, eR, ptL, ptR;
   {
@@ -1790,6 +1785,16 @@ __device__ void hlld_vjp(T gamma, const T* wl, const T* wr, T bn, const T* gf, T
   else
     fast_speed_vjp<T>(gamma, wr[0], wr[4], bn, wr[5], wr[6], gcmax, gwr[0], gwr[4], gbn_loc, gwr[5], gwr[6]);
   gbn += gbn_loc;
+}
+
+// Reverse of hlld(): gf = cotangent of the 7 flux components; accumulates
+// gwl[7], gwr[7] and gbn.  Follows the region selection, the degenerate
+// switches and the outer-speed selections of the forward solver.
+template <class T>
+__device__ void hlld_vjp(T gamma, const T* wl, const T* wr, T bn, const T* gf, T* gwl, T* gwr, T& gbn) {
+  const T gm1i = trcp<T>(gamma - T(1));
+  if constexpr (sizeof(T) != 4) hlld_diff_vjp<T>(gamma, gm1i, wl, wr, bn, gf, gwl, gwr, gbn);
+  else hlld_jump_vjp<T>(gamma, gm1i, wl, wr, bn, gf, gwl, gwr, gbn);
 }
 
 // ------------------------------------------------- primitive recovery VJP --

@@ -637,22 +637,22 @@ template <class T>
 __device__ __forceinline__ void hlld(T gamma, T gm1i, const T* wl, const T* wr, T bn, T* f) {
   if constexpr (sizeof(T) == 4) {
     hlld_jump<T>(gamma, gm1i, wl, wr, bn, f);
-    return;
-  }
-  TryOps<T> o;
-  hlld_diff<T>(o, gamma, gm1i, wl, wr, bn, f);
-  if constexpr (std::is_same<T, double>::value) {
-    if (__any_sync(__activemask(), o.bad)) {
-      if (o.bad) {
-        T a[7], b[7], c[7];
+  } else {
+    TryOps<T> o;
+    hlld_diff<T>(o, gamma, gm1i, wl, wr, bn, f);
+    if constexpr (std::is_same<T, double>::value) {
+      if (__any_sync(__activemask(), o.bad)) {
+        if (o.bad) {
+          T a[7], b[7], c[7];
 #pragma unroll
-        for (int q = 0; q < 7; ++q) {
-          a[q] = wl[q];
-          b[q] = wr[q];
+          for (int q = 0; q < 7; ++q) {
+            a[q] = wl[q];
+            b[q] = wr[q];
+          }
+          hlld_again<T>(gamma, gm1i, a, b, bn, c);
+#pragma unroll
+          for (int q = 0; q < 7; ++q) f[q] = c[q];
         }
-        hlld_again<T>(gamma, gm1i, a, b, bn, c);
-#pragma unroll
-        for (int q = 0; q < 7; ++q) f[q] = c[q];
       }
     }
   }
@@ -762,24 +762,8 @@ template <class T, class O> __device__ __forceinline__ EigCoef<T> eig_coef(O& o,
   }
   return C;
 }
-template <class T, class O>
-__device__ __forceinline__ void eig_left(O& o, const Eig<T>& E, const EigCoef<T>& C, const T* dw, T* q) {
-  if constexpr (sizeof(T) != 4) {
-    const T bv = times_sign<T>(o.mul(E.b1, dw[2]) + E.b2 * dw[3], E.sg);
-    const T bb = o.mul(E.b1, dw[5]) + E.b2 * dw[6];
-    const T Xf = o.mul(C.fp, dw[4]) + C.fb * bb, Yf = o.mul(C.su, bv) - C.fu * dw[1];
-    const T Xs = o.mul(C.sp, dw[4]) - C.sb * bb, Ys = o.mul(C.su, dw[1]) + C.fu * bv;
-    const T Z = o.mul(C.h1, dw[3]) - C.h2 * dw[2];
-    const T Zb = o.mul(C.z1, dw[6]) - C.z2 * dw[5];
-    q[0] = Xf + Yf;
-    q[1] = Z + Zb;
-    q[2] = Xs - Ys;
-    q[3] = dw[0] - dw[4] * E.ia2;
-    q[4] = Xs + Ys;
-    q[5] = Z - Zb;
-    q[6] = Xf - Yf;
-    return;
-  }
+// (float)
+template <class T> __device__ __forceinline__ void eig_left_narrow(const Eig<T>& E, const T* dw, T* q) {
   const T n = T(0.5) * E.ia2;
   const T ir = E.ir;
   const T bv = E.b1 * dw[2] + E.b2 * dw[3];
@@ -798,6 +782,26 @@ __device__ __forceinline__ void eig_left(O& o, const Eig<T>& E, const EigCoef<T>
   q[4] = n * (Xs - Ys);
   q[5] = Z - Zb;
   q[6] = n * (Xf - Yf);
+}
+template <class T, class O>
+__device__ __forceinline__ void eig_left(O& o, const Eig<T>& E, const EigCoef<T>& C, const T* dw, T* q) {
+  if constexpr (sizeof(T) != 4) {
+    const T bv = times_sign<T>(o.mul(E.b1, dw[2]) + E.b2 * dw[3], E.sg);
+    const T bb = o.mul(E.b1, dw[5]) + E.b2 * dw[6];
+    const T Xf = o.mul(C.fp, dw[4]) + C.fb * bb, Yf = o.mul(C.su, bv) - C.fu * dw[1];
+    const T Xs = o.mul(C.sp, dw[4]) - C.sb * bb, Ys = o.mul(C.su, dw[1]) + C.fu * bv;
+    const T Z = o.mul(C.h1, dw[3]) - C.h2 * dw[2];
+    const T Zb = o.mul(C.z1, dw[6]) - C.z2 * dw[5];
+    q[0] = Xf + Yf;
+    q[1] = Z + Zb;
+    q[2] = Xs - Ys;
+    q[3] = dw[0] - dw[4] * E.ia2;
+    q[4] = Xs + Ys;
+    q[5] = Z - Zb;
+    q[6] = Xf - Yf;
+  } else {
+    eig_left_narrow<T>(E, dw, q);
+  }
 }
 
 template <class T> __device__ __forceinline__ void eig_left(const Eig<T>& E, const EigCoef<T>& C, const T* dw, T* q) {
@@ -1083,11 +1087,7 @@ template <> __device__ __forceinline__ double ratio_any<double>(double a, double
 // multiplied, and sign flips and doublings are exact bit operations, so
 // only the arithmetic the limiter needs reaches the FP64 pipe.  Same values
 // as the formulas with q[2] kept, up to the sign of zero results.
-template <class T> __device__ __forceinline__ void ppm_one(const T* q, T& qm, T& qp) {
-  if constexpr (sizeof(T) != 4) {
-    ppm_one_wide<T>(q, qm, qp);
-    return;
-  }
+template <class T> __device__ __forceinline__ void ppm_one_narrow(const T* q, T& qm, T& qp) {
   const T c7 = from_d<T>(7.0 / 12.0), c1 = from_d<T>(1.0 / 12.0), c6 = from_d<T>(1.0 / 6.0);
   const T a = q[0], b = q[1], d = q[3], e = q[4];  // cells i-2, i-1, i+1, i+2
   qm = c7 * b - c1 * (a + d);
@@ -1123,6 +1123,11 @@ template <class T> __device__ __forceinline__ void ppm_one(const T* q, T& qm, T&
     if (abs_ge_twice<T>(qm, qp)) qm = neg<T>(twice_n<T>(qp));
     if (abs_ge_twice<T>(qp, m0)) qp = neg<T>(twice_n<T>(m0));
   }
+}
+
+template <class T> __device__ __forceinline__ void ppm_one(const T* q, T& qm, T& qp) {
+  if constexpr (sizeof(T) != 4) ppm_one_wide<T>(q, qm, qp);
+  else ppm_one_narrow<T>(q, qm, qp);
 }
 
 // The limiter as a call (double and float pairs): seven inlined copies outgrow
