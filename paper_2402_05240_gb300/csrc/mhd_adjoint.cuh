@@ -1102,7 +1102,7 @@ __device__ __forceinline__ void phys_cons_vjp(T gm1i, const T* w, T bn, const T*
 // reverse of the jump form, which carries both sides' star states and three
 // conserved vectors.  Measured: FP64 PPMC adjoint step at 128^3 55.7 -> 48.0 ms,
 // double-float rollout at 64^3 14.3 -> 10.8 ms (1 KB of register spill per
-// thread down to 0.1 KB).  The mass flux's rounding switch (rs == r) carries no
+// thread down to 0.45 KB, at 4 blocks per SM).  The mass flux's rounding switch (rs == r) carries no
 // derivative of its own.
 template <class T>
 __device__ __forceinline__ void hlld_diff_vjp(T gamma, T gm1i, const T* wl, const T* wr, T bn, const T* gf, T* gwl,

@@ -394,8 +394,8 @@ __global__ void __launch_bounds__(BX* BY) k_prim(Grid g, Fields<double, 8> U, Fi
     // range, not finite), can hold the grid's maximum.  Those cells evaluate
     // the rate in T: the maximum is that of the per-cell evaluation, bit for
     // bit, and most blocks evaluate none.  (k_prim<double> at 192^3: 1030 us with
-    // the library's reciprocal and the rate of each block's candidates, 399 us
-    // with both changed; 62 to 29 FP64-pipe slots per cell.)
+    // the library's reciprocal and the rate of each block's candidates, 342 us
+    // now; 62 to 25 FP64-pipe slots per cell.)
     if (dtbits) {
       auto in_range = [](double x) {  // 1e-9 <= x <= 1e9, on the bit pattern (integer pipes)
         const long long b = dbits(x);
@@ -494,8 +494,8 @@ template <class T> __device__ __forceinline__ void floor_face(const Grid& g, T* 
 // blocks of 128 threads per SM requested from the register allocator: 4 (at
 // most 128 registers per thread).  The float-pair kernels lose 9 % (PPMC) and
 // 12 % (PLMC) at 3 blocks, their dependent chains need the extra warps, and 7 %
-// and 1 % at 5 (spills); the double ones, which spill 0.2 KB at 4, lose 6 % and
-// 9 % at 3.
+// and 1 % at 5 (spills); the double ones, which spill 0.16 KB (PPMC) and 0.03 KB
+// (PLMC) at 4, lose 6 % and 9 % at 3.
 template <class T, int RECON> struct ReconMinBlocks { static constexpr int v = 4; };
 // interface states of cell p along A (Step 6): wl = W_{L,i+1/2} (the cell's
 // state at its upper face), wr = W_{R,i-1/2} (at its lower face), floored
@@ -902,10 +902,15 @@ __global__ void __launch_bounds__(BX* BY) k_update_half(Grid g, Fields<const dou
   const double h = S.h_half;
   // FP64: double differences; FP32-bulk and df half step: increments in T
   constexpr bool X = sizeof(T) == 8 && Exact<T>::full;
-  // (Faces, their stores, then the hydro update: the loads stay ordered against
-  // the stores, and this order holds the fewest values at a time.  256^3,
-  // FP32-bulk / float pairs: hydro first 0.915 / 1.295 ms, all stores last
-  // 0.846 / 1.284, this order 0.750 / 1.228 ms.)
+  // The loads stay ordered against the stores.  Faces, their stores, then the
+  // hydro update holds the fewest values at a time (256^3, FP32-bulk / float
+  // pairs: hydro first 0.915 / 1.295 ms, all stores last 0.846 / 1.284, this
+  // order 0.750 / 1.228 ms).  Double, bound by the FP64 pipe either way, loads
+  // for the hydro update first, which hides the latency of a grid of few blocks
+  // (20 steps of a 512 x 16 x 16 tube 12.78 -> 12.71 ms; 256^3 2.51 ms both).
+  constexpr bool kHydroFirst = std::is_same<T, double>::value;
+  double u5[5];
+  if constexpr (kHydroFirst) hydro_update<T, X, true>(U0, F, S, p, u5);
   // the cell's upper faces and its lower faces (the upper faces of p - e_a)
   const double bx = face_update<T, X, 0>(g, U0, E, h, c, p.m[1], p.m[2]);
   const double by = face_update<T, X, 1>(g, U0, E, h, c, p.m[2], p.m[0]);
@@ -916,8 +921,7 @@ __global__ void __launch_bounds__(BX* BY) k_update_half(Grid g, Fields<const dou
   Bh.f[0][c] = from_d<T>(bx);
   Bh.f[1][c] = from_d<T>(by);
   Bh.f[2][c] = from_d<T>(bz);
-  double u5[5];
-  hydro_update<T, X, true>(U0, F, S, p, u5);
+  if constexpr (!kHydroFirst) hydro_update<T, X, true>(U0, F, S, p, u5);
   // (the outer ghost layers of a padded grid see the wrap and carry no check)
   if ((!pos_bits(u5[0]) || !finite_bits(u5[4])) && interior(g, p.i, p.j, p.k)) atomicOr(flags, 1u);
   T w8[8];

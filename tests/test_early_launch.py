@@ -68,3 +68,34 @@ def test_replay_and_repeat(precision, n):
         s.synchronize()
     assert bool(torch.isfinite(A).all())
     assert torch.equal(A, B) and torch.equal(A, C)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", ["fp64", "fp64_df", "fp32_bulk"])
+def test_two_contexts_side_by_side(precision):
+    """Two contexts on two streams, their runs enqueued in turn, give the bits
+    of runs by themselves."""
+    import torch
+
+    from paper_2402_05240_gb300 import inputs as I
+    from paper_2402_05240_gb300 import mhd
+    shapes = [(33, 20, 17), (48, 9, 21)]
+    U0 = [torch.from_numpy(np.ascontiguousarray(I.turbulent_box(I.Box(*n), seed_v=3 + i, seed_b=4, kmax=4))).cuda()
+          for i, n in enumerate(shapes)]
+    alone = []
+    for n, u in zip(shapes, U0):
+        sim, A = mhd.Sim(*n, cfl=0.3, recon="ppmc", precision=precision), u.clone()
+        for _ in range(10):
+            sim.run(A, 3)
+        torch.cuda.synchronize()
+        alone.append(A)
+    streams = [torch.cuda.Stream() for _ in shapes]
+    sims = [mhd.Sim(*n, cfl=0.3, recon="ppmc", precision=precision, stream=s.cuda_stream)
+            for n, s in zip(shapes, streams)]
+    got = [u.clone() for u in U0]
+    torch.cuda.synchronize()
+    for _ in range(10):
+        for sim, A in zip(sims, got):
+            sim.run(A, 3)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(alone, got))
