@@ -83,26 +83,26 @@ ISSUE_PEAK_GWARPINST = 4 * 152 * 2.07
 # entry (its kernel was not captured).
 _STAGES = {
     "fp64": {
-        "prim": (21.0, 29.0, 893.1 / 32, 144.4),
-        "flux_pcm": (81.3, 117.4, 4006.7 / 32, 114.2),
-        "emf": (33.0, 33.0, 631.0 / 32, 118.3),
-        "update_half": (81.0, 116.0, 696.0 / 32, 315.6),
+        "prim": (21.0, 30.0, 889.8 / 32, 144.5),
+        "flux_pcm": (81.3, 117.4, 4006.7 / 32, 114.3),
+        "emf": (33.0, 33.0, 650.0 / 32, 118.4),
+        "update_half": (81.0, 117.0, 690.0 / 32, 315.5),
         "flux_hlld": (81.2, 117.2, 4015.1 / 32, 172.0),
         "update_full": (45.0, 66.0, 356.0 / 32, 268.5),
     },
     "fp32_bulk": {
-        "prim": (12.0, 18.0, 779.0 / 32, 102.5),
+        "prim": (12.0, 18.0, 785.0 / 32, 102.5),
         "flux_pcm": (0.0, 0.0, 495.3 / 32, 58.8),
         "emf": (0.0, 0.0, 223.0 / 32, 58.1),
-        "update_half": (23.0, 35.0, 1145.0 / 32, 188.5),
-        "flux_hlld": (0.0, 0.0, 526.2 / 32, 84.3),
+        "update_half": (23.0, 35.0, 1135.0 / 32, 188.6),
+        "flux_hlld": (0.0, 0.0, 526.2 / 32, 84.2),
         "update_full": (16.0, 19.0, 1049.1 / 32, 194.3),
     },
     "fp64_df": {
-        "prim": (15.0, 20.0, 952.5 / 32, 144.4),
-        "flux_pcm": (0.0, 0.0, 1987.3 / 32, 114.0),
+        "prim": (15.0, 21.0, 992.0 / 32, 144.4),
+        "flux_pcm": (0.0, 0.0, 1987.3 / 32, 114.1),
         "emf": (0.0, 0.0, 732.4 / 32, 118.2),
-        "update_half": (37.0, 48.0, 2019.0 / 32, 315.5),
+        "update_half": (37.0, 49.0, 2052.0 / 32, 315.6),
         "flux_hlld": (0.0, 0.0, 1970.7 / 32, 171.8),
         "update_full": (16.0, 19.0, 1096.0 / 32, 268.1),
     },
@@ -111,12 +111,12 @@ _STAGES = {
 # (sm__pipe_fp64_cycles_active, % of peak sustained active): the pipe's
 # occupancy by every FP64 instruction issued -- arithmetic, compares, and the
 # lanes a divergent branch leaves idle -- beside the algorithmic count above
-FP64_PIPE_BUSY = {"prim": 0.845, "flux_pcm": 0.802, "emf": 0.837, "update_half": 0.874, "recon": 0.842,
+FP64_PIPE_BUSY = {"prim": 0.844, "flux_pcm": 0.801, "emf": 0.836, "update_half": 0.874, "recon": 0.842,
                   "flux_hlld": 0.793, "update_full": 0.882}
 _RECON_PPMC = {
-    "fp64": (261.5, 348.3, 9340.4 / 32, 178.8),
+    "fp64": (259.5, 347.3, 9364.0 / 32, 181.2),
     "fp32_bulk": (0.0, 0.0, 1262.9 / 32, 80.9),
-    "fp64_df": (0.0, 0.0, 5313.3 / 32, 169.3),
+    "fp64_df": (0.0, 0.0, 5313.3 / 32, 169.4),
 }
 COUNTERS = {
     "plmc": {prec: dict(tab) for prec, tab in _STAGES.items()},
